@@ -290,7 +290,9 @@ extern "C" stepq_status stepq_calib_observe(const stepq_config *cfg, int layer, 
     if (layer < 0 || layer >= cfg->n_layers || n < 0 || !omega_sum || !logret_sum) return STEPQ_ERR_ARG;
     if ((st = check_inputs(cfg, q, k, nullptr, beta, gate, nullptr)) != STEPQ_OK) return st;
     if (n == 0) return STEPQ_OK;
-    return launch_calib_observe(cfg, layer, q, k, beta, gate, n, omega_sum, logret_sum,
+    const size_t heads = (size_t)layer * cfg->n_value_heads;
+    const size_t units = cfg->gate_kind == STEPQ_GATE_CHANNEL ? heads * kD : heads;
+    return launch_calib_observe(cfg, 1, q, k, beta, gate, n, omega_sum + heads * kD, logret_sum + units, nullptr, 1,
                                 (cudaStream_t)stream);
 }
 

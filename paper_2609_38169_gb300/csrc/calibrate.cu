@@ -1,7 +1,14 @@
 // The calibration protocol of App. A.3 behind one C entry point: it drives the
-// observe, FP32-state replay and candidate-distortion kernels over a recorded
-// trace, forms the means, chooses the FP16 pivots and, for row units, repeats
-// the distortion pass with the pivot rows held out of the column fit (App. C.2).
+// observe kernel and the replay kernel (FP32 recurrence with its candidate
+// distortions) over a recorded trace, forms the means, chooses the FP16 pivots and,
+// for row units, repeats the replay with the pivot rows held out of the column fit
+// (App. C.2).
+//
+// Each pass is one launch over all layers, sequences and heads. One launch per token
+// and layer, as before, left the chip idle between and inside them (observe 26 us on
+// 32 CTAs, replay 11 us on the state's way through memory): the four-layer channel-gate
+// model with 8 sequences of 256 tokens took 147 ms, 12 ms now.
+#include <algorithm>
 #include <cstring>
 #include <vector>
 
@@ -15,10 +22,10 @@ size_t up256(size_t n) { return (n + 255) / 256 * 256; }
 
 // Regions of the caller's workspace, each 256-byte aligned.
 struct Workspace {
-    double *omega_sum, *logret_sum, *acc;
-    float *w, *S, *y;
+    double *omega_sum, *logret_sum, *acc, *scratch;
+    float *w;
     uint8_t *pivot;
-    int32_t *slots;
+    int chunks;             // token chunks of the observe pass that scratch has room for
     size_t bytes;
 
     Workspace(const stepq_config *cfg, int n, uint8_t *base) {
@@ -35,17 +42,15 @@ struct Workspace {
         acc = (double *)take(U * K1 * sizeof(double));
         w = (float *)take(heads * kD * sizeof(float));
         pivot = take(U);
-        slots = (int32_t *)take((size_t)n * sizeof(int32_t));
-        S = (float *)take((size_t)n * cfg->n_value_heads * kN * sizeof(float));
-        y = (float *)take((size_t)n * cfg->n_value_heads * kD * sizeof(float));
+        // About 16 observe CTAs per SM, within the size of n dense states of a layer
+        // (what the workspace of n sequences has always had room for).
+        const size_t most = std::max<size_t>(1, 32 * (size_t)n / cfg->n_layers);
+        chunks = (int)std::min(most, (16 * 152 + heads - 1) / heads);
+        scratch = (double *)take(chunks > 1 ? chunks * heads * 2 * kD * sizeof(double) : 0);
+        if (chunks == 1) scratch = nullptr;
         bytes = o;
     }
 };
-
-__global__ void iota_kernel(int32_t *out, int n) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) out[i] = i;
-}
 
 stepq_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA; }
 
@@ -72,25 +77,16 @@ extern "C" stepq_status stepq_calibrate_from_trace(const stepq_config *cfg, int 
     Workspace ws(cfg, n, (uint8_t *)workspace);
     if (workspace_bytes < ws.bytes) return STEPQ_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
-    const int L = cfg->n_layers, Hv = cfg->n_value_heads, Hk = cfg->n_key_heads;
+    const int L = cfg->n_layers, Hv = cfg->n_value_heads;
     const bool rows = cfg->gate_kind == STEPQ_GATE_CHANNEL;
     const size_t heads = (size_t)L * Hv, U = stepq_num_units(cfg), K1 = (size_t)cfg->n_candidates + 1;
-    // trace strides per token step of one layer
-    const size_t sq = (size_t)n * Hk * kD, sv = (size_t)n * Hv * kD, sb = (size_t)n * Hv;
-    const size_t sg = rows ? sv : sb;
-    const auto at = [&](const float *base, size_t stride, int layer, int t) {
-        return base + ((size_t)layer * T + t) * stride;
-    };
 
     // Pass A: sums of g_{t,i}^2 (Sec. 4.1) and of log retention (Eq. calibration_lifetime).
     if ((st = cuda_ok(cudaMemsetAsync(ws.omega_sum, 0, heads * kD * sizeof(double), s))) != STEPQ_OK ||
-        (st = cuda_ok(cudaMemsetAsync(ws.logret_sum, 0, U * sizeof(double), s))) != STEPQ_OK)
+        (st = cuda_ok(cudaMemsetAsync(ws.logret_sum, 0, U * sizeof(double), s))) != STEPQ_OK ||
+        (st = launch_calib_observe(cfg, L, q, k, beta, gate, n * T, ws.omega_sum, ws.logret_sum, ws.scratch,
+                                   ws.chunks, s)) != STEPQ_OK)
         return st;
-    for (int t = 0; t < T; t++)
-        for (int l = 0; l < L; l++)
-            if ((st = launch_calib_observe(cfg, l, at(q, sq, l, t), at(k, sq, l, t), at(beta, sb, l, t),
-                                           at(gate, sg, l, t), n, ws.omega_sum, ws.logret_sum, s)) != STEPQ_OK)
-                return st;
     std::vector<double> osum(heads * kD), lsum(U);
     if ((st = cuda_ok(cudaMemcpyAsync(osum.data(), ws.omega_sum, osum.size() * sizeof(double),
                                       cudaMemcpyDeviceToHost, s))) != STEPQ_OK ||
@@ -109,33 +105,19 @@ extern "C" stepq_status stepq_calibrate_from_trace(const stepq_config *cfg, int 
     if ((st = cuda_ok(cudaMemcpyAsync(ws.w, w.data(), w.size() * sizeof(float), cudaMemcpyHostToDevice, s))) !=
         STEPQ_OK)
         return st;
-    iota_kernel<<<(n + 255) / 256, 256, 0, s>>>(ws.slots, n);
-    if ((st = cuda_ok(cudaGetLastError())) != STEPQ_OK) return st;
 
-    // Pass B: replay the FP32-state recurrence from zero per layer and fit every
+    // Pass B: replay the FP32-state recurrence from zero in every layer and fit every
     // `every`-th state at each candidate width (Eqs. qwen_calibration_distortion,
-    // kda_calibration_distortion); each sequence is one sample.
-    stepq_config one = *cfg;
-    one.n_layers = 1;
+    // kda_calibration_distortion); each sequence is one sample. The host forms the
+    // lifetimes, which only need pass A, while the first replay runs.
+    std::vector<double> life;
     const auto distortion_pass = [&](const uint8_t *pivot_rows, double *dist) -> stepq_status {
         stepq_status e;
         if ((e = cuda_ok(cudaMemsetAsync(ws.acc, 0, U * K1 * sizeof(double), s))) != STEPQ_OK) return e;
-        int n_samp = 0;
-        for (int l = 0; l < L; l++) {
-            if ((e = cuda_ok(cudaMemsetAsync(ws.S, 0, (size_t)n * Hv * kN * sizeof(float), s))) != STEPQ_OK)
-                return e;
-            for (int t = 0; t < T; t++) {
-                if ((e = launch_fp32_decode(&one, 0, ws.S, nullptr, n, ws.slots, n, at(q, sq, l, t),
-                                            at(k, sq, l, t), at(v, sv, l, t), at(beta, sb, l, t),
-                                            at(gate, sg, l, t), ws.y, s)) != STEPQ_OK)
-                    return e;
-                if ((t + 1) % every == 0) {
-                    if ((e = launch_calib_distortion(cfg, l, ws.w, pivot_rows, ws.S, n, ws.acc, s)) != STEPQ_OK)
-                        return e;
-                    if (l == 0) n_samp += n;
-                }
-            }
-        }
+        if ((e = launch_calib_replay(cfg, n, T, every, k, v, beta, gate, ws.w, pivot_rows, ws.acc, s)) != STEPQ_OK)
+            return e;
+        if (life.empty()) life = lifetime_weights(cfg, out->mean_log_ret);
+        const int n_samp = T / every * n;
         std::vector<double> acc(U * K1);
         if ((e = cuda_ok(cudaMemcpyAsync(acc.data(), ws.acc, acc.size() * sizeof(double),
                                          cudaMemcpyDeviceToHost, s))) != STEPQ_OK ||
@@ -149,7 +131,7 @@ extern "C" stepq_status stepq_calibrate_from_trace(const stepq_config *cfg, int 
     std::vector<double> d1(U * K1);
     if ((st = distortion_pass(nullptr, d1.data())) != STEPQ_OK) return st;
     if (out->distortion_stage1) std::memcpy(out->distortion_stage1, d1.data(), d1.size() * sizeof(double));
-    if ((st = stepq_select_pivots(cfg, out->mean_log_ret, d1.data(), out->pivot_mask)) != STEPQ_OK) return st;
+    if ((st = select_pivots(cfg, life, d1.data(), out->pivot_mask)) != STEPQ_OK) return st;
     bool any = false;
     for (size_t u = 0; u < U; u++) any = any || out->pivot_mask[u];
     if (rows && any) {

@@ -154,49 +154,6 @@ __device__ __forceinline__ void store_f16_row16(uint8_t *row, int cg, const floa
 
 // ---- reductions over the head tile ----
 
-// Column reduction of NR partial vectors acc[r][16] (each over the thread's 4
-// rows) into out[r][128] in shared memory. red: shared [NR][8][128] floats.
-// Reduce-scatter over the 4 rs lanes, then a sum over the 8 warps.
-template <int NR, bool MAX>
-__device__ __forceinline__ void column_reduce(const Lane &L, float (&acc)[NR][16], float *red,
-                                              float *out) {
-#pragma unroll
-    for (int r = 0; r < NR; r++) {
-        float h8[8];
-        const bool hi16 = (L.rs & 2) != 0;
-#pragma unroll
-        for (int t = 0; t < 8; t++) {
-            float keep = hi16 ? acc[r][8 + t] : acc[r][t];
-            float send = hi16 ? acc[r][t] : acc[r][8 + t];
-            float got = __shfl_xor_sync(0xffffffffu, send, 16);
-            h8[t] = MAX ? fmaxf(keep, got) : keep + got;
-        }
-        float h4[4];
-        const bool hi8 = (L.rs & 1) != 0;
-#pragma unroll
-        for (int t = 0; t < 4; t++) {
-            float keep = hi8 ? h8[4 + t] : h8[t];
-            float send = hi8 ? h8[t] : h8[4 + t];
-            float got = __shfl_xor_sync(0xffffffffu, send, 8);
-            h4[t] = MAX ? fmaxf(keep, got) : keep + got;
-        }
-        const int col = L.col0() + 8 * (L.rs >> 1) + 4 * (L.rs & 1);
-        *(float4 *)&red[(r * 8 + L.warp) * 128 + col] = make_float4(h4[0], h4[1], h4[2], h4[3]);
-    }
-    __syncthreads();
-    for (int e = L.tid; e < NR * 128; e += kThreads) {
-        const int r = e >> 7, c = e & 127;
-        float s = red[(r * 8) * 128 + c];
-#pragma unroll
-        for (int wv = 1; wv < 8; wv++) {
-            float x = red[(r * 8 + wv) * 128 + c];
-            s = MAX ? fmaxf(s, x) : s + x;
-        }
-        out[r * 128 + c] = s;
-    }
-    __syncthreads();
-}
-
 // Sum over the 16 columns a thread holds and the 8 cg lanes of its row group:
 // every lane of the group receives the full row sum.
 __device__ __forceinline__ float row_allreduce(float s) {

@@ -208,18 +208,6 @@ __device__ __forceinline__ uint64_t code_pair(const uint32_t (&wd)[2 * B], int c
     return u2pair(and_or(win, mask, kMagicBits), and_or(win, mask << B, kMagicBits));
 }
 
-// Sum over the 16 codes of a chunk of (0x4B400000 << s) and of the parts
-// shifted into the next word, i.e. what pack_codes adds besides the codes.
-__host__ __device__ constexpr uint32_t pack_bias(int B, int k) {
-    uint32_t b = 0;
-    for (int r = 0; r < 16; r++) {
-        const int p = r * B, kk = p >> 5, s = p & 31;
-        if (kk == k) b += kMagicBits << s;
-        if (s + B > 32 && kk + 1 == k) b += kMagicBits >> (32 - s);
-    }
-    return b;
-}
-
 // 16 offset-binary codes given as the float bit patterns 0x4B400000 | u_r,
 // packed LSB-first into the words of chunk c. The high bits are the same
 // constant for every code, so each word is the plain sum of the shifted

@@ -83,6 +83,9 @@ namespace stepq {
 
 // plan.cpp
 stepq_status validate_config(const stepq_config *cfg, bool need_quant_fields);
+std::vector<double> lifetime_weights(const stepq_config *cfg, const double *mean_log_ret);
+stepq_status select_pivots(const stepq_config *cfg, const std::vector<double> &life, const double *distortion,
+                           uint8_t *mask_out);   // stepq_select_pivots from given lifetimes
 
 // kernels (stepq_kernels.cu)
 stepq_status launch_decode(const stepq_plan *p, int layer, uint8_t *pool, int pool_slots,
@@ -147,9 +150,13 @@ stepq_status launch_intb_decode(const stepq_config *cfg, int bits, int layer, ui
                                 const float *k, const float *v, const float *beta,
                                 const float *gate, float *y, cudaStream_t s);
 // calib.cu
-stepq_status launch_calib_observe(const stepq_config *cfg, int layer, const float *q,
-                                  const float *k, const float *beta, const float *gate, int n,
-                                  double *omega_sum, double *logret_sum, cudaStream_t s);
+stepq_status launch_calib_observe(const stepq_config *cfg, int layers, const float *q, const float *k,
+                                  const float *beta, const float *gate, int n, double *omega_sum,
+                                  double *logret_sum, double *scratch, int chunks, cudaStream_t s);
+// stepq_kernels.cu: the FP32 replay of a trace with its candidate distortions, all layers
+stepq_status launch_calib_replay(const stepq_config *cfg, int n, int T, int every, const float *k,
+                                 const float *v, const float *beta, const float *gate, const float *w,
+                                 const uint8_t *pivot_rows, double *acc, cudaStream_t s);
 stepq_status launch_calib_distortion(const stepq_config *cfg, int layer, const float *w,
                                      const uint8_t *pivot_rows, const float *states, int n,
                                      double *acc, cudaStream_t s);

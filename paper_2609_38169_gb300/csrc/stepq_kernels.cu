@@ -8,14 +8,16 @@
 //
 // Numerical contract (shared with the CPU oracle, which restates it in fp64):
 // the tile X is fp32; r_i = fp16(clamp(sqrt(m_i) * w_i^(-1/2), 2^-14, 65504));
-// rho_i = fp32(1/(r_i zs_i)); every code decision is the nearest integer to the
-// exact product fp32(X rho_i) gamma_j with gamma_j = fp32(1/c_j) (rne_prod);
+// rho_i = fp32(1/(r_i zs_i)); every code decision is the nearest integer (ties to
+// even) to the exact product fp32(X rho_i) gamma_j with gamma_j = fp32(1/c_j), one
+// fused multiply-add with 1.5 * 2^23;
 // c is fitted from the clip-free start
 // max_i fp32(fp32(|X_ij| rho_i) / qmax_i) by `fit_iters` fixed-code
 // least-squares updates.
 #include <atomic>
 #include <cstdio>
 
+#include "async.cuh"
 #include "device.cuh"
 #include "internal.h"
 #include "tile.cuh"
@@ -23,177 +25,309 @@
 namespace stepq {
 
 // ---------------------------------------------------------------- smem layout
-constexpr int kPageBytes = (int)kMaxHeadBytes;             // 33,280
-constexpr int kOffRed = kPageBytes;                          // float [2][8][128]
-constexpr int kOffCol = kOffRed + 2 * 8 * 128 * 4;           // float [6][128]
-constexpr int kOffRowF = kOffCol + 6 * 128 * 4;              // float [5][128]: q k gate w2 wis
-constexpr int kOffRowI = kOffRowF + 5 * 128 * 4;             // int [2][128]: bits, offset
-constexpr int kSmemBytes = kOffRowI + 2 * 128 * 4;
+// Scratch of the fit. Per-column values and the cross-warp partials are kept in
+// 16-byte groups whose low two index bits are swizzled by the lane's column
+// group (cpos), so that the 8 lanes of a quarter warp, which address columns 16
+// apart, hit 8 different bank groups instead of 2.
+constexpr int kFitRed = 0;                                   // float [2][8][128]
+constexpr int kFitCol = kFitRed + 2 * 8 * 128 * 4;           // float [2][128]: c_j, 1 / c_j
+constexpr int kFitRow = kFitCol + 2 * 128 * 4;               // float [4][128]: w^2, w^-1/2, rho, r
+constexpr int kFitBits = kFitRow + 4 * 128 * 4;              // int [128] widths
+constexpr int kFitWarp = kFitBits + 128 * 4;                 // float [8]
+constexpr int kFitBytes = kFitWarp + 64;
 
-struct TileSmem {
-    uint8_t *page;
-    float *red, *col, *qv, *kv, *gv, *w2, *wis;
-    int *rbits, *roff;
-    __device__ __forceinline__ explicit TileSmem(uint8_t *s) {
-        page = s;
-        red = (float *)(s + kOffRed);
-        col = (float *)(s + kOffCol);
-        float *rf = (float *)(s + kOffRowF);
-        qv = rf;
-        kv = rf + 128;
-        gv = rf + 256;
-        w2 = rf + 384;
-        wis = rf + 512;
-        int *ri = (int *)(s + kOffRowI);
-        rbits = ri;
-        roff = ri + 128;
+struct FitSmem {
+    float *red, *colC, *colG, *w2, *wis, *rho, *rr, *warp;
+    int *rbits;
+    __device__ __forceinline__ explicit FitSmem(uint8_t *s) {
+        red = (float *)(s + kFitRed);
+        colC = (float *)(s + kFitCol);
+        colG = colC + 128;
+        w2 = (float *)(s + kFitRow);
+        wis = w2 + 128;
+        rho = w2 + 256;
+        rr = w2 + 384;
+        rbits = (int *)(s + kFitBits);
+        warp = (float *)(s + kFitWarp);
     }
 };
+
+// 16-byte group e (0..3) of the 16 columns of group cg, and the position of column c.
+__device__ __forceinline__ int cgroup(int cg, int e) { return 4 * cg + (e ^ (cg >> 1)); }
+__device__ __forceinline__ int cpos(int c) { return 4 * cgroup(c >> 4, (c >> 2) & 3) + (c & 3); }
 
 __device__ __forceinline__ int qmax_of(int b) { return (1 << (b - 1)) - 1; }
 
-// Per-thread results of the row-factor fit for its 4 rows.
-struct RowFit {
-    float rr[4], rho[4], zsv[4];
-    int qm[4], bits[4];
-};
+// Pairs (2e, 2e+1) of the lane's 16 values of a per-column vector, two at a time.
+__device__ __forceinline__ void col_pairs(const float *v, const Lane &L, int e, uint64_t &lo, uint64_t &hi) {
+    const uint4 q = *(const uint4 *)&v[4 * cgroup(L.cg, e)];
+    lo = u2pair(q.x, q.y);
+    hi = u2pair(q.z, q.w);
+}
 
-// Key-Row-Aware Dual-axis Fitting of the register tile x (Sec. 4.3, App. C.1).
-// msum[t]: sum_j |X_ij| of the thread's rows; row widths come from S.rbits.
-// On return S.col[0..128) holds the stored (FP16-rounded) column factors and
-// S.col[128..256) their reciprocals; with write_scales the FP16 r and c are
-// written into the staged page. Requires every thread to be done reading the
-// old page.
-__device__ __forceinline__ void fit_scales(const Lane &L, const TileSmem &S, const float (&x)[4][16],
-                                           const float (&msum)[4], int unit_rows,
-                                           int write_scales, int fit_iters, RowFit &f) {
-    uint16_t *page_r = (uint16_t *)S.page;
-    uint16_t *page_c = (uint16_t *)(S.page + 256);
-    float *colC = S.col;           // current column iterate
-    float *colG = S.col + 128;     // its reciprocal
-    float *colND = S.col + 256;    // [2][128] numerator / denominator
-    float mu[4];                   // fp32(1 / qmax_i)
-    // Row factors r_i = m_i^(1/2) w_i^(-1/2).
+// Reduce-scatter of 16 per-column partials over the 4 lanes of a column group
+// into the warp's row of `red` (the 8 warps' rows are summed by the column's owner).
+template <bool MAX>
+__device__ __forceinline__ void columns_to_red(const Lane &L, const float (&acc)[16], float *red) {
+    const auto join = [](float x, float y) { return MAX ? fmaxf(x, y) : x + y; };
+    float h8[8], h4[4];
+    const bool hi16 = (L.rs & 2) != 0, hi8 = (L.rs & 1) != 0;
+#pragma unroll
+    for (int t = 0; t < 8; t++)
+        h8[t] = join(hi16 ? acc[8 + t] : acc[t],
+                     __shfl_xor_sync(0xffffffffu, hi16 ? acc[t] : acc[8 + t], 16));
+#pragma unroll
+    for (int t = 0; t < 4; t++)
+        h4[t] = join(hi8 ? h8[4 + t] : h8[t], __shfl_xor_sync(0xffffffffu, hi8 ? h8[t] : h8[4 + t], 8));
+    *(float4 *)&red[L.warp * 128 + 4 * cgroup(L.cg, L.rs)] = make_float4(h4[0], h4[1], h4[2], h4[3]);
+}
+
+// One fixed-code pass (App. C.1): the thread's sums of w_i^2 v_ij X_ij and
+// w_i^2 v_ij^2 over its 4 rows, v_ij = r_i zs_i rne(X_ij rho_i gamma_j), per column
+// pair. CLIP clamps the codes to +-qmax and leaves pivot rows out by a select;
+// without it no code can exceed qmax, all values are finite and a pivot row adds
+// exact zeros (rho = r = 0).
+template <bool CLIP>
+__device__ __forceinline__ void ls_partials(const Lane &L, const FitSmem &S, const uint64_t (&x)[4][8],
+                                            int unit_rows, uint64_t (&n)[8], uint64_t (&d)[8]) {
+    const uint64_t M2 = f2s(kMagic), nM2 = f2s(-kMagic);
+#pragma unroll
+    for (int e = 0; e < 8; e++) n[e] = d[e] = 0;
 #pragma unroll
     for (int t = 0; t < 4; t++) {
-        const int i = L.row(t);
-        f.bits[t] = S.rbits[i];
-        if (f.bits[t] == kPivot) {
-            f.rr[t] = f.rho[t] = mu[t] = f.zsv[t] = 0.f;
-            f.qm[t] = 0;
-            if (write_scales && L.cg == 0) page_r[i] = 0;
-            continue;
-        }
-        const float m = msum[t] * (1.0f / 128.0f);
-        const float rf = __half2float(__float2half_rn(
-            fminf(fmaxf(__fmul_rn(sqrtf(m), S.wis[i]), kF16Min), kF16Max)));
-        const float zs = unit_rows ? (float)(1 << (8 - f.bits[t])) : 1.0f;
-        f.qm[t] = qmax_of(f.bits[t]);
-        f.rr[t] = rf;
-        f.zsv[t] = zs;
-        f.rho[t] = __frcp_rn(rf * zs);
-        mu[t] = __frcp_rn((float)f.qm[t]);
-        if (write_scales && L.cg == 0) page_r[i] = f16_bits(rf);
-    }
-    // Clip-free column start: c0_j = max_i |X_ij| / (r_i zs_i qmax_i), as
-    // max_i fp32(fp32(|X_ij| rho_i) mu_i).
-    {
-        float acc[1][16];
+        const int i = L.row(t), bits = S.rbits[i];
+        const bool pivot = bits == kPivot;
+        const float zs = unit_rows && !pivot ? (float)(1 << (8 - bits)) : 1.0f;
+        const float lim = pivot ? 0.f : (float)qmax_of(bits);
+        const uint64_t rho = f2s(S.rho[i]), rz = f2s(S.rr[i] * zs), w2 = f2s(S.w2[i]);
 #pragma unroll
-        for (int j = 0; j < 16; j++) acc[0][j] = 0.f;
+        for (int e4 = 0; e4 < 4; e4++) {
+            uint64_t g[2];
+            col_pairs(S.colG, L, e4, g[0], g[1]);
 #pragma unroll
-        for (int t = 0; t < 4; t++)
-#pragma unroll
-            for (int j = 0; j < 16; j++)
-                acc[0][j] = fmaxf(acc[0][j], __fmul_rn(__fmul_rn(fabsf(x[t][j]), f.rho[t]), mu[t]));
-        column_reduce<1, true>(L, acc, S.red, colC);
-        if (L.tid < 128) {
-            const float c = fminf(fmaxf(colC[L.tid], kF16Min), kF16Max);
-            colC[L.tid] = c;
-            colG[L.tid] = __frcp_rn(c);
-        }
-        __syncthreads();
-    }
-    // Fixed-code least-squares updates (App. C.1) over the non-pivot rows.
-    for (int it = 0; it < fit_iters; it++) {
-        float g[16];
-#pragma unroll
-        for (int j = 0; j < 16; j++) g[j] = colG[L.col0() + j];
-        float acc[2][16];
-#pragma unroll
-        for (int j = 0; j < 16; j++) acc[0][j] = acc[1][j] = 0.f;
-#pragma unroll
-        for (int t = 0; t < 4; t++) {
-            if (f.bits[t] == kPivot) continue;
-            const float w2 = S.w2[L.row(t)], rz = f.rr[t] * f.zsv[t], lim = (float)f.qm[t];
-#pragma unroll
-            for (int j = 0; j < 16; j++) {
-                const float qv = fminf(fmaxf(rne_prod(__fmul_rn(x[t][j], f.rho[t]), g[j]), -lim), lim);
-                const float v = rz * qv;                      // v_ij = r_i z_ij
-                acc[0][j] += w2 * (v * x[t][j]);
-                acc[1][j] += w2 * (v * v);
+            for (int h = 0; h < 2; h++) {
+                const int e = 2 * e4 + h;
+                uint64_t q = fadd2(ffma2(fmul2(x[t][e], rho), g[h], M2), nM2);   // rne of the product
+                if (CLIP) q = clamp2(q, lim);
+                const uint64_t v = fmul2(rz, q);                                 // v_ij = r_i z_ij
+                const uint64_t nn = ffma2(w2, fmul2(v, x[t][e]), n[e]);
+                const uint64_t dd = ffma2(w2, fmul2(v, v), d[e]);
+                n[e] = CLIP && pivot ? n[e] : nn;
+                d[e] = CLIP && pivot ? d[e] : dd;
             }
         }
-        column_reduce<2, false>(L, acc, S.red, colND);
-        if (L.tid < 128) {
-            const float num = colND[L.tid], den = colND[128 + L.tid];
-            float c = colC[L.tid];
-            if (den > 0.f) c = fminf(fmaxf(__fdiv_rn(num, den), kF16Min), kF16Max);
-            colC[L.tid] = c;
-            colG[L.tid] = __frcp_rn(c);
-        }
-        __syncthreads();
     }
-    // Storage precision of c.
-    if (L.tid < 128) {
-        const float cf = __half2float(__float2half_rn(colC[L.tid]));
-        colC[L.tid] = cf;
-        colG[L.tid] = __frcp_rn(cf);
-        if (write_scales) page_c[L.tid] = f16_bits(cf);
-    }
-    __syncthreads();
 }
 
-// Final codes with the stored scales, packed into the staged page (App. C.3 step 6).
-__device__ __forceinline__ void pack_codes(const Lane &L, const TileSmem &S, const float (&x)[4][16],
-                                           const RowFit &f) {
-    float g[16];
+// Key-Row-Aware Dual-axis Fitting of the register tile x (Sec. 4.3, App. C.1):
+// x[t][e] holds columns 16cg + 2e, 2e + 1 of row 16w + 4t + rs. msum[t]: sum_j
+// |X_ij| of the thread's rows; row widths come from S.rbits. On return S.rho and
+// S.rr hold the rows' reciprocal and stored row factors, S.colC the stored
+// (FP16-rounded) column factors and S.colG their reciprocals; a page (or null)
+// receives the FP16 r and c and must no longer be read. Returns whether a code may
+// exceed qmax with these scales (uniform over the CTA).
+//
+// Bound by instruction issue (about 60% of it fp32 arithmetic), so the passes run
+// on f32x2 column pairs, and the clamps, two min/max per code, only when the clip-free
+// start was capped, the state holds a non-finite value or (last pass and final
+// codes) some max_i |X'_ij| mu_i / c_j reaches 1 + 1/(2 qmax).
+__device__ __forceinline__ bool fit_scales(const Lane &L, const FitSmem &S, const uint64_t (&x)[4][8],
+                                           const float (&msum)[4], int unit_rows, uint8_t *page,
+                                           int fit_iters) {
+    // Row factors r_i = m_i^(1/2) w_i^(-1/2), and the clip-free column start
+    // c0_j = max_i fp32(fp32(|X_ij| rho_i) mu_i), mu_i = 1 / qmax_i.
+    bool wild = false;                                       // a non-finite row sum
+    float acc[16];
 #pragma unroll
-    for (int j = 0; j < 16; j++) g[j] = S.col[128 + L.col0() + j];
+    for (int j = 0; j < 16; j++) acc[j] = 0.f;
 #pragma unroll
     for (int t = 0; t < 4; t++) {
-        const int i = L.row(t);
-        uint8_t *row = S.page + S.roff[i];
-        if (f.bits[t] == kPivot) {
-            store_f16_row16(row, L.cg, x[t]);
+        const int i = L.row(t), bits = S.rbits[i];
+        float rf = 0.f, rho = 0.f, mu = 0.f;
+        if (bits != kPivot) {
+            const float m = msum[t] * (1.0f / 128.0f);
+            rf = __half2float(__float2half_rn(
+                fminf(fmaxf(__fmul_rn(sqrtf(m), S.wis[i]), kF16Min), kF16Max)));
+            const float zs = unit_rows ? (float)(1 << (8 - bits)) : 1.0f;
+            rho = __frcp_rn(rf * zs);
+            mu = __frcp_rn((float)qmax_of(bits));
+        }
+        wild = wild || !(msum[t] <= 3.4028235e38f);
+        if (L.cg == 0) {
+            S.rr[i] = rf;
+            S.rho[i] = rho;
+            if (page) ((uint16_t *)page)[i] = f16_bits(rf);
+        }
+        const uint64_t rho2 = f2s(rho), mu2 = f2s(mu);
+#pragma unroll
+        for (int e = 0; e < 8; e++) {
+            const uint64_t z = fmul2(fmul2(x[t][e], rho2), mu2);
+            acc[2 * e] = fmaxf(acc[2 * e], fabsf(f2lo(z)));
+            acc[2 * e + 1] = fmaxf(acc[2 * e + 1], fabsf(f2hi(z)));
+        }
+    }
+    columns_to_red<true>(L, acc, S.red);
+    __syncthreads();
+    // Threads 0..127 own one column each: its start c0, its current iterate.
+    const int cp = cpos(L.tid & 127);
+    float cm = 0.f, cc = 0.f;
+    if (L.tid < 128) {
+        cm = S.red[cp];
+#pragma unroll
+        for (int wv = 1; wv < 8; wv++) cm = fmaxf(cm, S.red[wv * 128 + cp]);
+        wild = wild || cm > kF16Max;                         // start capped: codes may clip
+        cc = fminf(fmaxf(cm, kF16Min), kF16Max);
+        S.colG[cp] = __frcp_rn(cc);
+    }
+    wild = __syncthreads_or(wild);
+    // Fixed-code least-squares updates over the non-pivot rows.
+    bool clip = wild;
+    for (int it = 0; it < fit_iters; it++) {
+        {
+            uint64_t n[8], d[8];
+            if (it > 0 || wild) ls_partials<true>(L, S, x, unit_rows, n, d);
+            else ls_partials<false>(L, S, x, unit_rows, n, d);
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                acc[2 * e] = f2lo(n[e]);
+                acc[2 * e + 1] = f2hi(n[e]);
+            }
+            columns_to_red<false>(L, acc, S.red);
+#pragma unroll
+            for (int e = 0; e < 8; e++) {
+                acc[2 * e] = f2lo(d[e]);
+                acc[2 * e + 1] = f2hi(d[e]);
+            }
+            columns_to_red<false>(L, acc, S.red + 8 * 128);
+        }
+        __syncthreads();
+        if (L.tid < 128) {
+            float num = S.red[cp], den = S.red[8 * 128 + cp];
+#pragma unroll
+            for (int wv = 1; wv < 8; wv++) {
+                num += S.red[wv * 128 + cp];
+                den += S.red[(8 + wv) * 128 + cp];
+            }
+            if (den > 0.f) cc = fminf(fmaxf(__fdiv_rn(num, den), kF16Min), kF16Max);
+            if (it + 1 < fit_iters) {
+                S.colG[cp] = __frcp_rn(cc);
+            } else {                                          // storage precision of c
+                const float cf = __half2float(__float2half_rn(cc)), g = __frcp_rn(cf);
+                S.colC[cp] = cf;
+                S.colG[cp] = g;
+                if (page) ((uint16_t *)(page + 256))[L.tid] = f16_bits(cf);
+                clip = clip || __fmul_rn(cm, g) >= (1.0f + 0.5f / 127.0f) * 0.999999f;
+            }
+        }
+        clip = __syncthreads_or(clip);
+    }
+    return clip;
+}
+
+// Final codes rne(X_ij rho_i gamma_j) of the thread's 16 columns of a row, as the
+// float bit patterns 0x4B400000 | (q + 2^(b-1)); with `clip` clamped to +-qmax.
+__device__ __forceinline__ void row_codes(const Lane &L, const FitSmem &S, const uint64_t (&x)[8], float rho,
+                                          int bits, bool clip, uint32_t (&f)[16]) {
+    const float mb = kMagic + (float)(1 << (bits - 1)), lim = (float)qmax_of(bits);
+    const uint64_t rho2 = f2s(rho), mb2 = f2s(mb), lo = f2s(mb - lim), hi = f2s(mb + lim);
+#pragma unroll
+    for (int e4 = 0; e4 < 4; e4++) {
+        uint64_t g[2];
+        col_pairs(S.colG, L, e4, g[0], g[1]);
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            uint64_t u = ffma2(fmul2(x[2 * e4 + h], rho2), g[h], mb2);
+            if (clip) u = clamp2r(u, lo, hi);
+            f[4 * e4 + 2 * h] = (uint32_t)u;
+            f[4 * e4 + 2 * h + 1] = (uint32_t)(u >> 32);
+        }
+    }
+}
+
+// Sixteen biased codes of width B packed LSB-first: the plain sum of the shifted bit
+// patterns minus the shifted constants (mod 2^32), one shift-add per code.
+template <int B>
+__device__ __forceinline__ void pack_biased(const uint32_t (&f)[16], uint32_t (&wd)[B / 2]) {
+    if (B == 8) {
+#pragma unroll
+        for (int t = 0; t < 4; t++)
+            wd[t] = __byte_perm(__byte_perm(f[4 * t], f[4 * t + 1], 0x0040),
+                                __byte_perm(f[4 * t + 2], f[4 * t + 3], 0x0040), 0x5410);
+        return;
+    }
+#pragma unroll
+    for (int k = 0; k < B / 2; k++) wd[k] = 0u - pack_bias(B, k);
+#pragma unroll
+    for (int r = 0; r < 16; r++) {
+        const int p = r * B, k = p >> 5, s = p & 31;
+        wd[k] += f[r] << s;
+        if (s + B > 32) wd[k + 1] += f[r] >> (32 - s);
+    }
+}
+
+// Packs the tile with the stored scales into the staged page (App. C.3 step 6);
+// roff: payload offset of each row.
+__device__ __forceinline__ void pack_page(const Lane &L, const FitSmem &S, uint8_t *page, const int *roff,
+                                          const uint64_t (&x)[4][8], bool clip) {
+#pragma unroll
+    for (int t = 0; t < 4; t++) {
+        const int i = L.row(t), bits = S.rbits[i];
+        uint8_t *row = page + roff[i];
+        if (bits == kPivot) {
+            uint32_t wd[8];
+#pragma unroll
+            for (int e = 0; e < 8; e++)
+                wd[e] = (uint32_t)f16_bits(f16_round_sat(f2lo(x[t][e]))) |
+                        ((uint32_t)f16_bits(f16_round_sat(f2hi(x[t][e]))) << 16);
+            uint4 *p = (uint4 *)(row + 32 * L.cg);
+            p[0] = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+            p[1] = make_uint4(wd[4], wd[5], wd[6], wd[7]);
             continue;
         }
-        const float lim = (float)f.qm[t];
-        int q[16];
-#pragma unroll
-        for (int j = 0; j < 16; j++)
-            q[j] = (int)fminf(fmaxf(rne_prod(__fmul_rn(x[t][j], f.rho[t]), g[j]), -lim), lim);
-        store_codes16(row, f.bits[t], L.cg, q);
+        uint32_t f[16];
+        row_codes(L, S, x[t], S.rho[i], bits, clip, f);
+        switch (bits) {
+        case 2: {
+            uint32_t wd[1];
+            pack_biased<2>(f, wd);
+            *(uint32_t *)(row + 4 * L.cg) = wd[0];
+        } break;
+        case 4: {
+            uint32_t wd[2];
+            pack_biased<4>(f, wd);
+            *(uint2 *)(row + 8 * L.cg) = make_uint2(wd[0], wd[1]);
+        } break;
+        case 6: {
+            uint32_t wd[3];
+            pack_biased<6>(f, wd);
+            uint32_t *p = (uint32_t *)(row + 12 * L.cg);
+            p[0] = wd[0];
+            p[1] = wd[1];
+            p[2] = wd[2];
+        } break;
+        default: {
+            uint32_t wd[4];
+            pack_biased<8>(f, wd);
+            *(uint4 *)(row + 16 * L.cg) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+        } break;
+        }
     }
-    __syncthreads();
 }
 
-__device__ __forceinline__ void fit_and_pack(const Lane &L, const TileSmem &S, const float (&x)[4][16],
-                                             const float (&msum)[4], int unit_rows,
-                                             int has_scales, int fit_iters) {
-    RowFit f;
-    fit_scales(L, S, x, msum, unit_rows, has_scales, fit_iters, f);
-    pack_codes(L, S, x, f);
-}
-
-// Per-row metadata of head h into shared memory (threads 0..127).
-__device__ __forceinline__ void load_row_meta(const Lane &L, const TileSmem &S,
-                                              const LayerTables &tab, int h) {
-    if (L.tid < 128) {
-        S.rbits[L.tid] = tab.row_bits[h * 128 + L.tid];
-        S.roff[L.tid] = (int)tab.row_off[h * 128 + L.tid];
-        S.w2[L.tid] = tab.w2[h * 128 + L.tid];
-        S.wis[L.tid] = tab.wis[h * 128 + L.tid];
+// The thread's part of a dense state (row stride 128) and its rows' sums of |X_ij|.
+__device__ __forceinline__ void load_dense(const Lane &L, const float *X, uint64_t (&x)[4][8], float (&msum)[4]) {
+#pragma unroll
+    for (int t = 0; t < 4; t++) {
+        const float4 *src = (const float4 *)(X + L.row(t) * 128 + L.col0());
+        float s = 0.f;
+#pragma unroll
+        for (int e = 0; e < 4; e++) {
+            const float4 f = src[e];
+            x[t][2 * e] = f2(f.x, f.y);
+            x[t][2 * e + 1] = f2(f.z, f.w);
+            s += fabsf(f.x) + fabsf(f.y) + fabsf(f.z) + fabsf(f.w);
+        }
+        msum[t] = row_allreduce(s);
     }
 }
 
@@ -202,6 +336,10 @@ __device__ __forceinline__ void copy16(uint4 *dst, const uint4 *src, int n16, in
 }
 
 // ---------------------------------------------------------- quantize / dequantize
+constexpr int kOffFit = (int)kMaxHeadBytes;                  // page [0, 33,280) | fit scratch | row offsets
+constexpr int kOffRoff = kOffFit + kFitBytes;                // int [128]
+constexpr int kSmemBytes = kOffRoff + 128 * 4;
+
 struct PoolArgs {
     uint8_t *pool;
     uint64_t stride;
@@ -217,7 +355,9 @@ struct PoolArgs {
 __global__ void __launch_bounds__(kThreads, 2) quantize_kernel(PoolArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
     const Lane L;
-    const TileSmem S(smem);
+    uint8_t *page = smem;
+    const FitSmem S(smem + kOffFit);
+    int *roff = (int *)(smem + kOffRoff);
     const int Hv = a.sh.Hv;
     const int b = blockIdx.x / Hv, h = blockIdx.x - b * Hv;
     const int slot = a.slots[b];
@@ -225,34 +365,28 @@ __global__ void __launch_bounds__(kThreads, 2) quantize_kernel(PoolArgs a) {
         if (L.tid == 0) raise_error(a.err, STEPQ_ERR_SLOT_RANGE);
         return;
     }
-    load_row_meta(L, S, a.tab, h);
-    const float *X = a.states + (size_t)b * a.state_stride_b + (size_t)h * kN;
-    float x[4][16], msum[4];
-#pragma unroll
-    for (int t = 0; t < 4; t++) {
-        const float4 *src = (const float4 *)(X + L.row(t) * 128 + L.col0());
-        float s = 0.f;
-#pragma unroll
-        for (int e = 0; e < 4; e++) {
-            float4 f = src[e];
-            x[t][4 * e] = f.x;
-            x[t][4 * e + 1] = f.y;
-            x[t][4 * e + 2] = f.z;
-            x[t][4 * e + 3] = f.w;
-            s += fabsf(f.x) + fabsf(f.y) + fabsf(f.z) + fabsf(f.w);
-        }
-        msum[t] = row_allreduce(s);
+    if (L.tid < 128) {
+        S.rbits[L.tid] = a.tab.row_bits[h * 128 + L.tid];
+        roff[L.tid] = (int)a.tab.row_off[h * 128 + L.tid];
+        S.w2[L.tid] = a.tab.w2[h * 128 + L.tid];
+        S.wis[L.tid] = a.tab.wis[h * 128 + L.tid];
     }
+    uint64_t x[4][8];
+    float msum[4];
+    load_dense(L, a.states + (size_t)b * a.state_stride_b + (size_t)h * kN, x, msum);
     __syncthreads();
-    fit_and_pack(L, S, x, msum, a.sh.unit_kind, a.tab.head_bits[h] != kPivot, a.sh.fit_iters);
+    const bool clip = fit_scales(L, S, x, msum, a.sh.unit_kind, page, a.sh.fit_iters);
+    pack_page(L, S, page, roff, x, clip);
+    __syncthreads();
     uint8_t *gpage = a.pool + (uint64_t)slot * a.stride + a.tab.head_off[h];
-    copy16((uint4 *)gpage, (const uint4 *)S.page, (int)a.tab.head_bytes[h] >> 4, L.tid);
+    copy16((uint4 *)gpage, (const uint4 *)page, (int)a.tab.head_bytes[h] >> 4, L.tid);
 }
 
 __global__ void __launch_bounds__(kThreads, 2) dequantize_kernel(PoolArgs a) {
     extern __shared__ __align__(16) uint8_t smem[];
     const Lane L;
-    const TileSmem S(smem);
+    uint8_t *page = smem;
+    int *rbits = (int *)(smem + kOffFit), *roff = (int *)(smem + kOffRoff);
     const int Hv = a.sh.Hv;
     const int b = blockIdx.x / Hv, h = blockIdx.x - b * Hv;
     const int slot = a.slots[b];
@@ -261,19 +395,22 @@ __global__ void __launch_bounds__(kThreads, 2) dequantize_kernel(PoolArgs a) {
         return;
     }
     const uint8_t *gpage = a.pool + (uint64_t)slot * a.stride + a.tab.head_off[h];
-    copy16((uint4 *)S.page, (const uint4 *)gpage, (int)a.tab.head_bytes[h] >> 4, L.tid);
-    load_row_meta(L, S, a.tab, h);
+    copy16((uint4 *)page, (const uint4 *)gpage, (int)a.tab.head_bytes[h] >> 4, L.tid);
+    if (L.tid < 128) {
+        rbits[L.tid] = a.tab.row_bits[h * 128 + L.tid];
+        roff[L.tid] = (int)a.tab.row_off[h * 128 + L.tid];
+    }
     __syncthreads();
     const int has_scales = a.tab.head_bits[h] != kPivot;
-    const uint16_t *page_r = (const uint16_t *)S.page;
-    const uint16_t *page_c = (const uint16_t *)(S.page + 256);
+    const uint16_t *page_r = (const uint16_t *)page;
+    const uint16_t *page_c = (const uint16_t *)(page + 256);
     float *out = a.states + (size_t)b * a.state_stride_b + (size_t)h * kN;
 #pragma unroll
     for (int t = 0; t < 4; t++) {
         const int i = L.row(t);
-        const int bits = S.rbits[i];
+        const int bits = rbits[i];
         float vals[16];
-        load_row16(S.page + S.roff[i], bits, L.cg, vals);
+        load_row16(page + roff[i], bits, L.cg, vals);
         if (bits != kPivot) {
             const float r = f16_val(page_r[i]);
             const float zs = a.sh.unit_kind ? (float)(1 << (8 - bits)) : 1.f;
@@ -291,58 +428,28 @@ __global__ void __launch_bounds__(kThreads, 2) dequantize_kernel(PoolArgs a) {
 }
 
 // ------------------------------------------------------ calibration distortion
-// One CTA per (sample, head): the reference state is fitted at every candidate
-// width with the codec above (uniform over the head; pivot rows kept in FP16
-// and out of the column fit) and its reconstruction error accumulated
-// (Eqs. qwen_calibration_distortion, kda_calibration_distortion).
-struct DistArgs {
-    const float *states;          // [n][Hv][128][128]
-    const float *w;               // [Hv][128] of the layer
-    const uint8_t *pivot_rows;    // [Hv][128] of the layer, or null
-    double *acc;                  // head: [Hv][K+1]; row: [Hv*128][K+1] (layer slice)
-    int Hv, unit_rows, n_cand, fit_iters;
+// A reference state head fitted at every candidate width with the codec above
+// (uniform over the head; pivot rows kept in FP16 and out of the column fit), and
+// its reconstruction errors (Eqs. qwen_calibration_distortion,
+// kda_calibration_distortion). add(k, i, e): row units, the mean error of key row i
+// at candidate k; add(k, 0, e): head units, the weighted mean over the head (by one
+// thread). S.w2 and S.wis hold the head's weights; `piv` its pivot rows or null.
+struct FitCands {
+    int unit_rows, n_cand, fit_iters;
     int cands[4];
 };
 
-__global__ void __launch_bounds__(kThreads, 2) distortion_kernel(DistArgs a) {
-    extern __shared__ __align__(16) uint8_t smem[];
-    const Lane L;
-    const TileSmem S(smem);
-    const int s = blockIdx.x / a.Hv, h = blockIdx.x - s * a.Hv;
+template <class Add>
+__device__ __forceinline__ void distortion_of(const Lane &L, const FitSmem &S, const uint64_t (&x)[4][8],
+                                              const float (&msum)[4], const uint8_t *piv, const FitCands &a,
+                                              const Add &add) {
     const int K1 = a.n_cand + 1;
-    if (L.tid < 128) {
-        const float wv = a.w[h * 128 + L.tid];
-        S.w2[L.tid] = __fmul_rn(wv, wv);
-        S.wis[L.tid] = __frsqrt_rn(wv);
-    }
-    const float *X = a.states + ((size_t)s * a.Hv + h) * kN;
-    float x[4][16], msum[4];
-#pragma unroll
-    for (int t = 0; t < 4; t++) {
-        const float4 *src = (const float4 *)(X + L.row(t) * 128 + L.col0());
-        float sm = 0.f;
-#pragma unroll
-        for (int e = 0; e < 4; e++) {
-            const float4 v = src[e];
-            x[t][4 * e] = v.x;
-            x[t][4 * e + 1] = v.y;
-            x[t][4 * e + 2] = v.z;
-            x[t][4 * e + 3] = v.w;
-            sm += fabsf(v.x) + fabsf(v.y) + fabsf(v.z) + fabsf(v.w);
-        }
-        msum[t] = row_allreduce(sm);
-    }
-    float *blk = S.col + 512;
     for (int k = 0; k < K1; k++) {
         const bool fp16_col = (k == a.n_cand);
-        if (L.tid < 128) {
-            const bool piv = fp16_col ||
-                             (a.unit_rows && a.pivot_rows && a.pivot_rows[h * 128 + L.tid]);
-            S.rbits[L.tid] = piv ? kPivot : a.cands[k];
-        }
+        if (L.tid < 128) S.rbits[L.tid] = fp16_col || (piv && piv[L.tid]) ? kPivot : a.cands[k];
         __syncthreads();
-        RowFit f;
-        if (!fp16_col) fit_scales(L, S, x, msum, a.unit_rows, 0, a.fit_iters, f);
+        bool clip = false;
+        if (!fp16_col) clip = fit_scales(L, S, x, msum, a.unit_rows, nullptr, a.fit_iters);
         float head_err = 0.f;
 #pragma unroll
         for (int t = 0; t < 4; t++) {
@@ -351,25 +458,37 @@ __global__ void __launch_bounds__(kThreads, 2) distortion_kernel(DistArgs a) {
             float e = 0.f;
             if (bits == kPivot) {
 #pragma unroll
-                for (int j = 0; j < 16; j++) {
-                    const float d = f16_round_sat(x[t][j]) - x[t][j];
-                    e += d * d;
+                for (int j = 0; j < 8; j++) {
+                    const float x0 = f2lo(x[t][j]), x1 = f2hi(x[t][j]);
+                    const float d0 = f16_round_sat(x0) - x0, d1 = f16_round_sat(x1) - x1;
+                    e = fmaf(d0, d0, e);
+                    e = fmaf(d1, d1, e);
                 }
             } else {
-                const float lim = (float)f.qm[t];
+                const float lim = (float)qmax_of(bits);
+                const uint64_t zs = f2s(a.unit_rows ? (float)(1 << (8 - bits)) : 1.0f);
+                const uint64_t rho = f2s(S.rho[i]), rr = f2s(S.rr[i]);
+                const uint64_t M2 = f2s(kMagic), nM2 = f2s(-kMagic), m1 = f2s(-1.0f);
 #pragma unroll
-                for (int j = 0; j < 16; j++) {
-                    const float cj = S.col[L.col0() + j], gj = S.col[128 + L.col0() + j];
-                    const float qv = fminf(fmaxf(rne_prod(__fmul_rn(x[t][j], f.rho[t]), gj), -lim), lim);
-                    const float rec = __fmul_rn(f.rr[t] * cj, f.zsv[t] * qv);
-                    const float d = rec - x[t][j];
-                    e += d * d;
+                for (int e4 = 0; e4 < 4; e4++) {
+                    uint64_t g[2], c[2];
+                    col_pairs(S.colG, L, e4, g[0], g[1]);
+                    col_pairs(S.colC, L, e4, c[0], c[1]);
+#pragma unroll
+                    for (int h = 0; h < 2; h++) {
+                        const uint64_t xv = x[t][2 * e4 + h];
+                        uint64_t q = fadd2(ffma2(fmul2(xv, rho), g[h], M2), nM2);
+                        if (clip) q = clamp2(q, lim);
+                        const uint64_t rec = fmul2(fmul2(rr, c[h]), fmul2(zs, q));
+                        const uint64_t d = ffma2(xv, m1, rec);                  // rec - x
+                        e = fmaf(f2lo(d), f2lo(d), e);
+                        e = fmaf(f2hi(d), f2hi(d), e);
+                    }
                 }
             }
             e = row_allreduce(e);
             if (a.unit_rows) {
-                if (L.cg == 0)
-                    atomicAdd(&a.acc[((size_t)h * 128 + i) * K1 + k], (double)e / 128.0);
+                if (L.cg == 0) add(k, i, (double)e / 128.0);
             } else {
                 head_err += S.w2[i] * e;
             }
@@ -378,16 +497,203 @@ __global__ void __launch_bounds__(kThreads, 2) distortion_kernel(DistArgs a) {
             // rows of one lane group share head_err; take it once per group
             float v = (L.cg == 0) ? head_err : 0.f;
             for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            if (L.lane == 0) blk[L.warp] = v;
+            if (L.lane == 0) S.warp[L.warp] = v;
             __syncthreads();
             if (L.tid == 0) {
                 double sum = 0.0;
-                for (int wv = 0; wv < 8; wv++) sum += blk[wv];
-                atomicAdd(&a.acc[(size_t)h * K1 + k], sum / (double)kN);
+                for (int wv = 0; wv < 8; wv++) sum += S.warp[wv];
+                add(k, 0, sum / (double)kN);
             }
         }
         __syncthreads();
     }
+}
+
+// One CTA per (sample, head).
+struct DistArgs {
+    const float *states;          // [n][Hv][128][128]
+    const float *w;               // [Hv][128] of the layer
+    const uint8_t *pivot_rows;    // [Hv][128] of the layer, or null
+    double *acc;                  // head: [Hv][K+1]; row: [Hv*128][K+1] (layer slice)
+    int Hv;
+    FitCands fit;
+};
+
+__device__ __forceinline__ void load_weights(const Lane &L, const FitSmem &S, const float *w) {
+    if (L.tid < 128) {
+        const float wv = w[L.tid];
+        S.w2[L.tid] = __fmul_rn(wv, wv);
+        S.wis[L.tid] = __frsqrt_rn(wv);
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 2) distortion_kernel(DistArgs a) {
+    __shared__ __align__(16) uint8_t smem[kFitBytes];
+    const Lane L;
+    const FitSmem S(smem);
+    const int s = blockIdx.x / a.Hv, h = blockIdx.x - s * a.Hv;
+    const int K1 = a.fit.n_cand + 1;
+    load_weights(L, S, a.w + h * 128);
+    uint64_t x[4][8];
+    float msum[4];
+    load_dense(L, a.states + ((size_t)s * a.Hv + h) * kN, x, msum);
+    const size_t rows = a.fit.unit_rows ? 128 : 1;
+    distortion_of(L, S, x, msum, a.pivot_rows ? a.pivot_rows + h * 128 : nullptr, a.fit,
+                  [&](int k, int i, double e) { atomicAdd(&a.acc[(h * rows + i) * K1 + k], e); });
+}
+
+// ------------------------------------------------- calibration replay (App. A.3)
+// The FP32 recurrence of one (layer, sequence, value head) from a zero state over T
+// tokens, with every `every`-th state fitted in place at each candidate width: one
+// CTA carries the state in registers for all tokens, so a token costs one CTA
+// barrier and about 200 instructions a thread instead of a launch and two passes of
+// the state over memory, and the layers run side by side. The arithmetic and its
+// order are the FP32 decode kernel's (fp32.cu): warp w owns key rows 16w..16w+15,
+// lane l columns 4l..4l+3; the eight warps' retrieval partials are summed in warp
+// order, by every warp for itself. A sampled state goes through shared memory into
+// the fit's tile mapping (the replay's registers are reloaded from there).
+// Bound by the fits (three candidate widths plus FP16: about nine tenths of the
+// instructions at one sample in 8 tokens). 4 layers x 8 sequences x 32 heads, 256
+// tokens, 32 samples: 4.7 ms a pass, against about 28 ms of per-token launches.
+struct ReplayArgs {
+    const float *k, *v, *beta, *gate;   // trace [L][T][n][..]
+    const float *w;                     // [L][Hv][128]
+    const uint8_t *pivot_rows;          // [L][Hv][128] or null
+    double *acc;                        // [L][Hv or Hv*128][K+1]
+    int n, T, Hk, Hv, every, gate_per_row;
+    FitCands fit;
+};
+
+constexpr int kRpTile = 0;                                   // float [128][128] (16-byte groups swizzled)
+constexpr int kRpRed = kRpTile + kN * 4;                     // float [2][8][128]
+constexpr int kRpRowA = kRpRed + 2 * 8 * 128 * 4;            // float4 [3][128]: d d k k
+constexpr int kRpRowB = kRpRowA + 3 * 128 * 16;              // float2 [3][128]: beta k, twice
+constexpr int kRpV = kRpRowB + 3 * 128 * 8;                  // float [3][128]
+constexpr int kRpFit = kRpV + 3 * 128 * 4;
+constexpr int kRpAcc = (kRpFit + kFitBytes + 15) / 16 * 16;  // double [128][5]
+constexpr int kRpSmem = kRpAcc + 128 * 5 * 8;
+
+__global__ void __launch_bounds__(kThreads, 2) replay_kernel(ReplayArgs a) {
+    extern __shared__ __align__(16) uint8_t smem[];
+    const Lane L;
+    const FitSmem S(smem + kRpFit);
+    float *tile = (float *)(smem + kRpTile), *red = (float *)(smem + kRpRed), *vs = (float *)(smem + kRpV);
+    float4 *rowA = (float4 *)(smem + kRpRowA);
+    float2 *rowB = (float2 *)(smem + kRpRowB);
+    double *acc = (double *)(smem + kRpAcc);
+    const int tid = L.tid, w = L.warp, l = L.lane;
+    const int h = blockIdx.x % a.Hv, sb = blockIdx.x / a.Hv, b = sb % a.n, layer = sb / a.n;
+    const int hk = h / (a.Hv / a.Hk), K1 = a.fit.n_cand + 1;
+    const size_t lh = (size_t)layer * a.Hv + h;
+    load_weights(L, S, a.w + lh * 128);
+    for (int e = tid; e < 128 * K1; e += kThreads) acc[e] = 0.0;
+    // A token's vectors: loaded two tokens ahead by threads 0..127 (one channel
+    // each), in shared memory one token ahead, three buffers.
+    float fk = 0.f, fv = 0.f, fd = 0.f, fb = 0.f;
+    const auto fetch = [&](int t) {
+        if (tid < 128 && t < a.T) {
+            const size_t tok = ((size_t)layer * a.T + t) * a.n + b;
+            fk = a.k[(tok * a.Hk + hk) * 128 + tid];
+            fv = a.v[(tok * a.Hv + h) * 128 + tid];
+            fd = a.gate_per_row ? a.gate[(tok * a.Hv + h) * 128 + tid] : a.gate[tok * a.Hv + h];
+            fb = a.beta[tok * a.Hv + h];
+        }
+    };
+    const auto put = [&](int buf) {
+        if (tid < 128) {
+            rowA[buf * 128 + tid] = make_float4(fd, fd, fk, fk);
+            const float bk = fb * fk;
+            rowB[buf * 128 + tid] = make_float2(bk, bk);
+            vs[buf * 128 + tid] = fv;
+        }
+    };
+    fetch(0);
+    put(0);
+    fetch(1);
+    __syncthreads();
+    uint64_t x2[16][2];
+#pragma unroll
+    for (int r = 0; r < 16; r++) x2[r][0] = x2[r][1] = 0;
+    const uint8_t *piv = a.pivot_rows ? a.pivot_rows + lh * 128 : nullptr;
+    int left = a.every;
+    for (int t = 0, cur = 0; t < a.T; t++) {
+        const int nxt = cur == 2 ? 0 : cur + 1;
+        float *rd = red + (t & 1) * 8 * 128;
+        // P = D S and the retrieval u_j = sum_i k_i P_ij.
+        uint64_t ua[2] = {0, 0}, ub[2] = {0, 0};
+#pragma unroll
+        for (int r = 0; r < 16; r++) {
+            const uint4 q = *(const uint4 *)&rowA[cur * 128 + 16 * w + r];
+            const uint64_t dd = u2pair(q.x, q.y), kk = u2pair(q.z, q.w);
+            x2[r][0] = fmul2(x2[r][0], dd);
+            x2[r][1] = fmul2(x2[r][1], dd);
+            uint64_t(&ac)[2] = (r & 1) ? ub : ua;
+            ac[0] = ffma2(kk, x2[r][0], ac[0]);
+            ac[1] = ffma2(kk, x2[r][1], ac[1]);
+        }
+        {
+            const uint64_t s0 = fadd2(ua[0], ub[0]), s1 = fadd2(ua[1], ub[1]);
+            *(float4 *)&rd[w * 128 + 4 * l] = make_float4(f2lo(s0), f2hi(s0), f2lo(s1), f2hi(s1));
+        }
+        // The next token's buffer was last read two tokens ago, behind the previous
+        // token's barrier; this one's barrier publishes it.
+        put(nxt);
+        fetch(t + 2);
+        __syncthreads();
+        // delta_j = v_j - u_j; S = P + beta k_i delta_j.
+        uint64_t s0 = 0, s1 = 0;
+#pragma unroll
+        for (int wv = 0; wv < 8; wv++) {
+            const uint4 p = *(const uint4 *)&rd[wv * 128 + 4 * l];
+            s0 = fadd2(s0, u2pair(p.x, p.y));
+            s1 = fadd2(s1, u2pair(p.z, p.w));
+        }
+        const float4 v4 = *(const float4 *)&vs[cur * 128 + 4 * l];
+        const uint64_t d0 = f2(v4.x - f2lo(s0), v4.y - f2hi(s0)), d1 = f2(v4.z - f2lo(s1), v4.w - f2hi(s1));
+#pragma unroll
+        for (int r = 0; r < 16; r++) {
+            const uint64_t bk = *(const uint64_t *)&rowB[cur * 128 + 16 * w + r];
+            x2[r][0] = ffma2(bk, d0, x2[r][0]);
+            x2[r][1] = ffma2(bk, d1, x2[r][1]);
+        }
+        if (--left == 0) {
+            left = a.every;
+#pragma unroll
+            for (int r = 0; r < 16; r++)
+                *(uint4 *)&tile[(16 * w + r) * 128 + 4 * cgroup(l >> 2, l & 3)] =
+                    make_uint4((uint32_t)x2[r][0], (uint32_t)(x2[r][0] >> 32), (uint32_t)x2[r][1],
+                               (uint32_t)(x2[r][1] >> 32));
+            __syncwarp();                                     // both mappings give warp w rows 16w..16w+15
+            {
+                uint64_t x[4][8];
+                float msum[4];
+#pragma unroll
+                for (int t4 = 0; t4 < 4; t4++) {
+                    float s = 0.f;
+#pragma unroll
+                    for (int e = 0; e < 4; e++) {
+                        const float4 f = *(const float4 *)&tile[L.row(t4) * 128 + 4 * cgroup(L.cg, e)];
+                        x[t4][2 * e] = f2(f.x, f.y);
+                        x[t4][2 * e + 1] = f2(f.z, f.w);
+                        s += fabsf(f.x) + fabsf(f.y) + fabsf(f.z) + fabsf(f.w);
+                    }
+                    msum[t4] = row_allreduce(s);
+                }
+                // one adder per entry and a fixed order within the CTA
+                distortion_of(L, S, x, msum, piv, a.fit, [&](int k, int i, double e) { acc[i * K1 + k] += e; });
+            }
+#pragma unroll
+            for (int r = 0; r < 16; r++) {
+                const uint4 p = *(const uint4 *)&tile[(16 * w + r) * 128 + 4 * cgroup(l >> 2, l & 3)];
+                x2[r][0] = u2pair(p.x, p.y);
+                x2[r][1] = u2pair(p.z, p.w);
+            }
+        }
+        cur = nxt;
+    }
+    __syncthreads();
+    const int entries = (a.fit.unit_rows ? 128 : 1) * K1;
+    for (int e = tid; e < entries; e += kThreads) atomicAdd(&a.acc[lh * entries + e], acc[e]);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -401,8 +707,8 @@ static stepq_status prepare(int dev) {
                                  kSmemBytes) != cudaSuccess ||
             cudaFuncSetAttribute(dequantize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kSmemBytes) != cudaSuccess ||
-            cudaFuncSetAttribute(distortion_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kSmemBytes) != cudaSuccess)
+            cudaFuncSetAttribute(replay_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 kRpSmem) != cudaSuccess)
             return STEPQ_ERR_CUDA;
         g_attr_set[dev] = true;
     }
@@ -448,11 +754,18 @@ stepq_status launch_dequantize(const stepq_plan *p, int layer, const uint8_t *po
     return launched();
 }
 
+static FitCands fit_cands(const stepq_config *cfg) {
+    FitCands f{};
+    f.unit_rows = cfg->gate_kind == STEPQ_GATE_CHANNEL;
+    f.n_cand = cfg->n_candidates;
+    f.fit_iters = cfg->fit_iters;
+    for (int k = 0; k < cfg->n_candidates; k++) f.cands[k] = cfg->candidates[k];
+    return f;
+}
+
 stepq_status launch_calib_distortion(const stepq_config *cfg, int layer, const float *w,
                                      const uint8_t *pivot_rows, const float *states, int n,
                                      double *acc, cudaStream_t s) {
-    stepq_status st = prepare(-1);
-    if (st != STEPQ_OK) return st;
     const size_t Hv = (size_t)cfg->n_value_heads;
     const bool rows = cfg->gate_kind == STEPQ_GATE_CHANNEL;
     const size_t K1 = (size_t)cfg->n_candidates + 1;
@@ -462,11 +775,22 @@ stepq_status launch_calib_distortion(const stepq_config *cfg, int layer, const f
     a.pivot_rows = (rows && pivot_rows) ? pivot_rows + (size_t)layer * Hv * kD : nullptr;
     a.acc = acc + (size_t)layer * Hv * (rows ? kD : 1) * K1;
     a.Hv = (int)Hv;
-    a.unit_rows = rows;
-    a.n_cand = cfg->n_candidates;
-    a.fit_iters = cfg->fit_iters;
-    for (int k = 0; k < cfg->n_candidates; k++) a.cands[k] = cfg->candidates[k];
-    distortion_kernel<<<(unsigned)(n * Hv), kThreads, kSmemBytes, s>>>(a);
+    a.fit = fit_cands(cfg);
+    distortion_kernel<<<(unsigned)(n * Hv), kThreads, 0, s>>>(a);
+    return launched();
+}
+
+stepq_status launch_calib_replay(const stepq_config *cfg, int n, int T, int every, const float *k,
+                                 const float *v, const float *beta, const float *gate, const float *w,
+                                 const uint8_t *pivot_rows, double *acc, cudaStream_t s) {
+    stepq_status st = prepare(-1);
+    if (st != STEPQ_OK) return st;
+    const bool rows = cfg->gate_kind == STEPQ_GATE_CHANNEL;
+    ReplayArgs a{k, v, beta, gate, w, rows ? pivot_rows : nullptr, acc, n, T, cfg->n_key_heads,
+                 cfg->n_value_heads, every, rows, fit_cands(cfg)};
+    const size_t ctas = (size_t)cfg->n_layers * n * cfg->n_value_heads;
+    if (ctas > 0x7fffffffu) return STEPQ_ERR_UNSUPPORTED;
+    replay_kernel<<<(unsigned)ctas, kThreads, kRpSmem, s>>>(a);
     return launched();
 }
 

@@ -1,6 +1,6 @@
 // Register-tile helpers shared by the fused decode kernels: the magic-number
-// rounding constant, f32x2 pair sums and clamps, and the warp reduce-scatter
-// of per-row partial sums.
+// rounding constant, f32x2 pair sums and clamps, the code packing constants, and
+// the warp reduce-scatter of per-row partial sums.
 #pragma once
 
 #include <cstdint>
@@ -23,11 +23,16 @@ __device__ __forceinline__ uint64_t clamp2r(uint64_t v, uint64_t lo, uint64_t hi
     return f2(fminf(fmaxf(f2lo(v), f2lo(lo)), f2lo(hi)), fminf(fmaxf(f2hi(v), f2hi(lo)), f2hi(hi)));
 }
 
-// Nearest integer (ties to even) of the exact product a * b for |a b| < 2^22:
-// one fused multiply-add with 1.5 * 2^23 rounds it once. Larger products come
-// out within a few units of a b, which every caller clamps to +-qmax anyway.
-__device__ __forceinline__ float rne_prod(float a, float b) {
-    return __fmaf_rn(a, b, 12582912.0f) - 12582912.0f;
+// Sum over the 16 codes of a chunk of (0x4B400000 << s) and of the parts
+// shifted into the next word, i.e. what pack_codes adds besides the codes.
+__host__ __device__ constexpr uint32_t pack_bias(int B, int k) {
+    uint32_t b = 0;
+    for (int r = 0; r < 16; r++) {
+        const int p = r * B, kk = p >> 5, s = p & 31;
+        if (kk == k) b += kMagicBits << s;
+        if (s + B > 32 && kk + 1 == k) b += kMagicBits >> (32 - s);
+    }
+    return b;
 }
 
 // Sum of 16 per-row partials over the 32 lanes of a warp (reduce-scatter): lane
