@@ -39,15 +39,7 @@ extern "C" stepq_status stepq_quantize_pool(const stepq_plan *p, int layer, cons
     if (!states) return STEPQ_ERR_ARG;
     if (!aligned(states, 16)) return STEPQ_ERR_ALIGN;
     if (B == 0) return STEPQ_OK;
-    const size_t per_layer = (size_t)p->cfg.n_value_heads * kN;
-    cudaStream_t s = (cudaStream_t)stream;
-    if (layer >= 0) return launch_quantize(p, layer, states, per_layer, slots, B, (uint8_t *)pool, pool_slots, s);
-    for (int l = 0; l < p->cfg.n_layers; l++) {
-        st = launch_quantize(p, l, states + l * per_layer, per_layer * p->cfg.n_layers, slots, B,
-                             (uint8_t *)pool, pool_slots, s);
-        if (st != STEPQ_OK) return st;
-    }
-    return STEPQ_OK;
+    return launch_quantize(p, layer, states, slots, B, (uint8_t *)pool, pool_slots, (cudaStream_t)stream);
 }
 
 extern "C" stepq_status stepq_dequantize_pool(const stepq_plan *p, int layer, const void *pool,
@@ -58,15 +50,7 @@ extern "C" stepq_status stepq_dequantize_pool(const stepq_plan *p, int layer, co
     if (!states) return STEPQ_ERR_ARG;
     if (!aligned(states, 16)) return STEPQ_ERR_ALIGN;
     if (B == 0) return STEPQ_OK;
-    const size_t per_layer = (size_t)p->cfg.n_value_heads * kN;
-    cudaStream_t s = (cudaStream_t)stream;
-    if (layer >= 0) return launch_dequantize(p, layer, (const uint8_t *)pool, pool_slots, slots, B, states, per_layer, s);
-    for (int l = 0; l < p->cfg.n_layers; l++) {
-        st = launch_dequantize(p, l, (const uint8_t *)pool, pool_slots, slots, B,
-                               states + l * per_layer, per_layer * p->cfg.n_layers, s);
-        if (st != STEPQ_OK) return st;
-    }
-    return STEPQ_OK;
+    return launch_dequantize(p, layer, (const uint8_t *)pool, pool_slots, slots, B, states, (cudaStream_t)stream);
 }
 
 extern "C" size_t stepq_temporal_slot_bytes(const stepq_plan *p) { return p ? p->t_slot_stride : 0; }

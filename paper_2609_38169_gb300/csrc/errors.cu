@@ -34,6 +34,19 @@ unsigned int *device_error_word() {
     return (unsigned int *)symbol_address((const void *)&g_error_word, addr);
 }
 
+int sm_count() {
+    static std::atomic<int> n[64];        // per device; racing first calls store the same value
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) return 1;
+    int v = n[dev].load(std::memory_order_relaxed);
+    if (!v) {
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+        n[dev].store(v, std::memory_order_relaxed);
+    }
+    return v > 0 ? v : 1;
+}
+
 // The pipelined kernels' wait bound and withheld item (test support). Plain
 // process-wide values: stepq_debug_stall is documented as not thread-safe.
 static long long g_wait_cycles = pipe::kWaitCycles;

@@ -25,8 +25,6 @@
 // memory, and a bulk store writes it back. CTA barriers per item: one after the
 // row constants (which also agrees on the stage's copies), two around the row
 // factors, one before the store.
-#include <atomic>
-
 #include "async.cuh"
 #include "device.cuh"
 #include "internal.h"
@@ -659,7 +657,7 @@ struct PoolArgs {
     uint64_t stride;
     int pool_slots;
     const int32_t *slots;
-    int Hv;
+    int heads, items;          // heads per batch entry (one layer's or all layers'); item = entry * heads + head
     LayerTables tab;
     float *states;
     size_t state_stride_b;
@@ -667,101 +665,148 @@ struct PoolArgs {
     int fit_iters;
 };
 
+// Pack of dense states, persistent, two CTAs per SM. Once an item's tile is in
+// registers its shared-memory copy is refilled with the next item's state (16-byte
+// cp.async), so the loads run under the fit, and the page leaves by a bulk store.
+// (One CTA per item with plain loads was stalled on them half of the time: 106 us for
+// 4096 heads at 6 bits, 60 us now; 47 us at the copy rate of HBM.) The 16-byte
+// groups of a row are swizzled by its band, so that the 8 lanes of a quarter warp,
+// which read one column quad of 8 bands, hit 8 bank groups.
 constexpr int kPageMaxHead = 32768;
-constexpr int kPoolSmem = kOffStages + kPageMaxHead + kVecBytes;
-
-template <int B>
-__device__ __forceinline__ void quantize_item(const T &t, const Smem &S, uint8_t *page, const float *w2,
-                                              const float *wis, const float *X, int fit_iters) {
-    uint64_t x2[8][4];
-    float rs[16];
-#pragma unroll
-    for (int m = 0; m < 8; m++) {
-        const float4 r0 = *(const float4 *)(X + t.row(2 * m) * 128 + t.col(0));
-        const float4 r1 = *(const float4 *)(X + t.row(2 * m + 1) * 128 + t.col(0));
-        x2[m][0] = f2(r0.x, r1.x);
-        x2[m][1] = f2(r0.y, r1.y);
-        x2[m][2] = f2(r0.z, r1.z);
-        x2[m][3] = f2(r0.w, r1.w);
-        abs_row_sums(x2[m], rs[2 * m], rs[2 * m + 1]);
-    }
-    if constexpr (B == kPivot) {
-        pack_pivot(t, page, x2, 1.f);
-    } else {
-        fit_pack<B>(t, S, page, w2, wis, false, x2, rs, fit_iters, [] {});
-    }
-}
+constexpr int kOffQTile = kOffStages;
+constexpr int kOffQPage = kOffQTile + kN * 4;
+constexpr int kOffQVec = kOffQPage + kPageMaxHead;        // float [2][128]: w^2, w^-1/2
+constexpr int kPackSmem = kOffQVec + 2 * 128 * 4;
+__device__ __forceinline__ int tile_at(int row, int f) { return row * 128 + 4 * (f ^ ((row >> 4) & 7)); }
 
 __global__ void __launch_bounds__(kThreads, 2) quantize_heads_kernel(PoolArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     const T t;
     const Smem S(smem);
-    const int b = blockIdx.x / a.Hv, h = blockIdx.x - b * a.Hv;
-    const int slot = a.slots[b];
-    if (slot < 0 || slot >= a.pool_slots) {
-        if (t.tid == 0) raise_error(a.err, STEPQ_ERR_SLOT_RANGE);
-        return;
+    float *tile = (float *)(smem + kOffQTile), *w2 = (float *)(smem + kOffQVec), *wis = w2 + 128;
+    uint8_t *page = smem + kOffQPage;
+    const auto slot_of = [&](int item) { return item < a.items ? a.slots[item / a.heads] : -1; };
+    const auto ok = [&](int slot) { return slot >= 0 && slot < a.pool_slots; };
+    float fw2 = 0.f, fwis = 0.f;
+    const auto start = [&](int item) {
+        const int b = item / a.heads, h = item - b * a.heads;
+        const float4 *X = (const float4 *)(a.states + (size_t)b * a.state_stride_b + (size_t)h * kN);
+#pragma unroll
+        for (int j = 0; j < 16; j++) {
+            const int e = t.tid + j * kThreads;
+            cp_async16(&tile[tile_at(e >> 5, e & 31)], X + e);
+        }
+        if (t.tid < 128) {
+            fw2 = a.tab.w2[h * 128 + t.tid];
+            fwis = a.tab.wis[h * 128 + t.tid];
+        }
+    };
+    int slot = slot_of(blockIdx.x);
+    if (ok(slot)) start(blockIdx.x);
+    for (int item = blockIdx.x; item < a.items; item += gridDim.x) {
+        const int next = item + gridDim.x, nslot = slot_of(next);
+        if (!ok(slot)) {                                  // uniform over the CTA
+            if (t.tid == 0) raise_error(a.err, STEPQ_ERR_SLOT_RANGE);
+            if (ok(nslot)) start(next);
+            slot = nslot;
+            continue;
+        }
+        const int h = item % a.heads, bits = a.tab.head_bits[h];
+        if (t.tid < 128) {
+            w2[t.tid] = fw2;
+            wis[t.tid] = fwis;
+        }
+        cp_async_wait_all();
+        __syncthreads();
+        uint64_t x2[8][4];
+        float rs[16];
+#pragma unroll
+        for (int m = 0; m < 8; m++) {
+            const float4 r0 = *(const float4 *)&tile[tile_at(t.row(2 * m), 4 * t.w + t.cg)];
+            const float4 r1 = *(const float4 *)&tile[tile_at(t.row(2 * m + 1), 4 * t.w + t.cg)];
+            x2[m][0] = f2(r0.x, r1.x);
+            x2[m][1] = f2(r0.y, r1.y);
+            x2[m][2] = f2(r0.z, r1.z);
+            x2[m][3] = f2(r0.w, r1.w);
+            abs_row_sums(x2[m], rs[2 * m], rs[2 * m + 1]);
+        }
+        if (t.tid == 0) bulk_wait_read_all();             // the previous page has left
+        __syncthreads();
+        if (ok(nslot)) start(next);
+        switch (bits) {
+        case 2: fit_pack<2>(t, S, page, w2, wis, false, x2, rs, a.fit_iters, [] {}); break;
+        case 4: fit_pack<4>(t, S, page, w2, wis, false, x2, rs, a.fit_iters, [] {}); break;
+        case 6: fit_pack<6>(t, S, page, w2, wis, false, x2, rs, a.fit_iters, [] {}); break;
+        case 8: fit_pack<8>(t, S, page, w2, wis, false, x2, rs, a.fit_iters, [] {}); break;
+        default: pack_pivot(t, page, x2, 1.f); break;
+        }
+        fence_async_smem();
+        __syncthreads();
+        if (t.tid == 0) {
+            bulk_store(a.pool + (uint64_t)slot * a.stride + a.tab.head_off[h], page, a.tab.head_bytes[h]);
+            bulk_commit();
+        }
+        slot = nslot;
     }
-    uint8_t *page = S.stages;
-    float *w2 = (float *)(page + kPageMaxHead), *wis = w2 + 128;
-    if (t.tid < 128) {
-        w2[t.tid] = a.tab.w2[h * 128 + t.tid];
-        wis[t.tid] = a.tab.wis[h * 128 + t.tid];
-    }
-    __syncthreads();
-    const float *X = a.states + (size_t)b * a.state_stride_b + (size_t)h * kN;
-    switch (a.tab.head_bits[h]) {
-    case 2: quantize_item<2>(t, S, page, w2, wis, X, a.fit_iters); break;
-    case 4: quantize_item<4>(t, S, page, w2, wis, X, a.fit_iters); break;
-    case 6: quantize_item<6>(t, S, page, w2, wis, X, a.fit_iters); break;
-    case 8: quantize_item<8>(t, S, page, w2, wis, X, a.fit_iters); break;
-    default: quantize_item<kPivot>(t, S, page, w2, wis, X, a.fit_iters); break;
-    }
-    __syncthreads();
-    uint8_t *gpage = a.pool + (uint64_t)slot * a.stride + a.tab.head_off[h];
-    const int n16 = (int)a.tab.head_bytes[h] >> 4;
-    for (int e = t.tid; e < n16; e += kThreads) ((uint4 *)gpage)[e] = ((const uint4 *)page)[e];
+    if (t.tid == 0) bulk_wait_all();
 }
 
+// Dense tile of an unpacked page in shared memory: a band of 16 rows is 8 KB, as in
+// the dense state, and 16 bytes of padding (the 8 lanes of a quarter warp store one
+// column quad of the 8 bands: 8 bank groups).
+constexpr int kBandBytes = 16 * 512 + 16;
+constexpr int kUnpackSmem = 8 * kBandBytes;
+
 template <int B>
-__device__ __forceinline__ void dequantize_item(const T &t, const uint8_t *page, float *out) {
+__device__ __forceinline__ void dequantize_item(const T &t, const uint8_t *page, uint8_t *tile) {
     uint64_t x2[8][4];
     load_tile<B>(t, page, x2);      // c_j q_ij (exact) or the FP16 value
     const uint16_t *page_r = (const uint16_t *)page;
+    float4 *out = (float4 *)(tile + t.rg * kBandBytes) + 4 * t.w + t.cg;
 #pragma unroll
     for (int m = 0; m < 8; m++) {
         // r_i c_j z_ij rounded once: c_j q_ij is exact in fp32 (fp16 x 8 bits)
-        const uint64_t rr = B == kPivot ? 0 : f2(f16_val(page_r[t.row(2 * m)]), f16_val(page_r[t.row(2 * m + 1)]));
+        const uint32_t rp = B == kPivot ? 0u : *(const uint32_t *)(page_r + t.row(2 * m));
+        const uint64_t rr = f2(f16_val((uint16_t)(rp & 0xFFFFu)), f16_val((uint16_t)(rp >> 16)));
         uint64_t v[4];
 #pragma unroll
         for (int c = 0; c < 4; c++) v[c] = B == kPivot ? x2[m][c] : fmul2(rr, x2[m][c]);
-        *(float4 *)(out + t.row(2 * m) * 128 + t.col(0)) = make_float4(f2lo(v[0]), f2lo(v[1]), f2lo(v[2]), f2lo(v[3]));
-        *(float4 *)(out + t.row(2 * m + 1) * 128 + t.col(0)) = make_float4(f2hi(v[0]), f2hi(v[1]), f2hi(v[2]), f2hi(v[3]));
+        out[64 * m] = make_float4(f2lo(v[0]), f2lo(v[1]), f2lo(v[2]), f2lo(v[3]));
+        out[64 * m + 32] = make_float4(f2hi(v[0]), f2hi(v[1]), f2hi(v[2]), f2hi(v[3]));
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 2) dequantize_heads_kernel(PoolArgs a) {
+// Unpack, one CTA per (slot, head) and bound by the 64 KB it writes. The page's
+// streams are interleaved over a warp's lanes, so a thread reads its pieces straight
+// from the page in whole 512-byte requests; the dense rows, of which a warp holds 64
+// bytes each, meet in shared memory and leave as one 8 KB bulk store a band. (Staging
+// the page first and storing the 64-byte pieces took 98 us for 4096 heads at 6 bits,
+// direct reads with those stores 73 us, this form 53 us; 47 us at the copy rate of
+// HBM.)
+__global__ void __launch_bounds__(kThreads, 3) dequantize_heads_kernel(PoolArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];
     const T t;
-    const Smem S(smem);
-    const int b = blockIdx.x / a.Hv, h = blockIdx.x - b * a.Hv;
+    const int b = blockIdx.x / a.heads, h = blockIdx.x - b * a.heads;
     const int slot = a.slots[b];
     if (slot < 0 || slot >= a.pool_slots) {
         if (t.tid == 0) raise_error(a.err, STEPQ_ERR_SLOT_RANGE);
         return;
     }
-    uint8_t *page = S.stages;
-    const uint8_t *gpage = a.pool + (uint64_t)slot * a.stride + a.tab.head_off[h];
-    const int n16 = (int)a.tab.head_bytes[h] >> 4;
-    for (int e = t.tid; e < n16; e += kThreads) ((uint4 *)page)[e] = ((const uint4 *)gpage)[e];
-    __syncthreads();
+    const uint8_t *page = a.pool + (uint64_t)slot * a.stride + a.tab.head_off[h];
     float *out = a.states + (size_t)b * a.state_stride_b + (size_t)h * kN;
     switch (a.tab.head_bits[h]) {
-    case 2: dequantize_item<2>(t, page, out); break;
-    case 4: dequantize_item<4>(t, page, out); break;
-    case 6: dequantize_item<6>(t, page, out); break;
-    case 8: dequantize_item<8>(t, page, out); break;
-    default: dequantize_item<kPivot>(t, page, out); break;
+    case 2: dequantize_item<2>(t, page, smem); break;
+    case 4: dequantize_item<4>(t, page, smem); break;
+    case 6: dequantize_item<6>(t, page, smem); break;
+    case 8: dequantize_item<8>(t, page, smem); break;
+    default: dequantize_item<kPivot>(t, page, smem); break;
+    }
+    fence_async_smem();
+    __syncthreads();
+    if (t.tid < 8) {
+        bulk_store(out + t.tid * 16 * 128, smem + t.tid * kBandBytes, 16 * 512);
+        bulk_commit();
+        bulk_wait_read_all();                             // shared memory outlives the reads
     }
 }
 
@@ -772,19 +817,6 @@ static stepq_status set_attr(const void *fn, int bytes) {
     return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess
                ? STEPQ_OK
                : STEPQ_ERR_CUDA;
-}
-
-static int sm_count() {
-    static std::atomic<int> n[64];        // per device; racing first calls store the same value
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) return 1;
-    int v = n[dev].load(std::memory_order_relaxed);
-    if (!v) {
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
-        n[dev].store(v, std::memory_order_relaxed);
-    }
-    return v > 0 ? v : 1;
 }
 
 stepq_status launch_decode_heads(const stepq_plan *p, int layer, uint8_t *pool, int pool_slots,
@@ -838,37 +870,27 @@ stepq_status launch_decode_heads_mode(const stepq_plan *p, int layer, uint8_t *p
     return cudaGetLastError() == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
 }
 
-static hk::PoolArgs pool_args(const stepq_plan *p, int layer, uint8_t *pool, int pool_slots,
-                              const int32_t *slots, float *states, size_t stride_b) {
-    hk::PoolArgs a{};
-    a.pool = pool;
-    a.stride = p->slot_stride;
-    a.pool_slots = pool_slots;
-    a.slots = slots;
-    a.Hv = p->cfg.n_value_heads;
-    a.tab = p->layer(layer);
-    a.states = states;
-    a.state_stride_b = stride_b;
-    a.err = device_error_word();
-    a.fit_iters = p->cfg.fit_iters;
-    return a;
+static hk::PoolArgs pool_args(const stepq_plan *p, int layer, const float *states, const int32_t *slots, int B,
+                              uint8_t *pool, int pool_slots) {
+    const int heads = p->cfg.n_value_heads * (layer < 0 ? p->cfg.n_layers : 1);
+    return {pool, p->slot_stride, pool_slots, slots, heads, B * heads, p->layer(layer < 0 ? 0 : layer),
+            (float *)states, (size_t)heads * kN, device_error_word(), p->cfg.fit_iters};
 }
 
-stepq_status launch_quantize_heads(const stepq_plan *p, int layer, const float *states,
-                                   size_t stride_b, const int32_t *slots, int B, uint8_t *pool,
-                                   int pool_slots, cudaStream_t s) {
-    if (set_attr((const void *)hk::quantize_heads_kernel, hk::kPoolSmem) != STEPQ_OK) return STEPQ_ERR_CUDA;
-    hk::PoolArgs a = pool_args(p, layer, pool, pool_slots, slots, (float *)states, stride_b);
-    hk::quantize_heads_kernel<<<(unsigned)B * a.Hv, kThreads, hk::kPoolSmem, s>>>(a);
+stepq_status launch_quantize_heads(const stepq_plan *p, int layer, const float *states, const int32_t *slots,
+                                   int B, uint8_t *pool, int pool_slots, cudaStream_t s) {
+    if (set_attr((const void *)hk::quantize_heads_kernel, hk::kPackSmem) != STEPQ_OK) return STEPQ_ERR_CUDA;
+    const hk::PoolArgs a = pool_args(p, layer, states, slots, B, pool, pool_slots);
+    const int grid = 2 * sm_count();
+    hk::quantize_heads_kernel<<<grid < a.items ? grid : a.items, kThreads, hk::kPackSmem, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
 }
 
-stepq_status launch_dequantize_heads(const stepq_plan *p, int layer, const uint8_t *pool,
-                                     int pool_slots, const int32_t *slots, int B, float *states,
-                                     size_t stride_b, cudaStream_t s) {
-    if (set_attr((const void *)hk::dequantize_heads_kernel, hk::kPoolSmem) != STEPQ_OK) return STEPQ_ERR_CUDA;
-    hk::PoolArgs a = pool_args(p, layer, (uint8_t *)pool, pool_slots, slots, states, stride_b);
-    hk::dequantize_heads_kernel<<<(unsigned)B * a.Hv, kThreads, hk::kPoolSmem, s>>>(a);
+stepq_status launch_dequantize_heads(const stepq_plan *p, int layer, const uint8_t *pool, int pool_slots,
+                                     const int32_t *slots, int B, float *states, cudaStream_t s) {
+    if (set_attr((const void *)hk::dequantize_heads_kernel, hk::kUnpackSmem) != STEPQ_OK) return STEPQ_ERR_CUDA;
+    const hk::PoolArgs a = pool_args(p, layer, states, slots, B, (uint8_t *)pool, pool_slots);
+    hk::dequantize_heads_kernel<<<a.items, kThreads, hk::kUnpackSmem, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
 }
 

@@ -29,13 +29,6 @@ struct LayerTables {
     const uint32_t *row_slot; // [Hv][128] s-th stored row: offset | width << 16 | row << 24
 };
 
-struct Shape {
-    int Hk, Hv, n_layers;
-    int gate_per_row;         // 1 for the channel gate (KDA)
-    int unit_kind;            // 0 head units, 1 row units
-    int fit_iters;
-};
-
 }  // namespace stepq
 
 struct stepq_plan {
@@ -72,11 +65,6 @@ struct stepq_plan {
                 d_head_bytes + l * Hv, d_head_bits + l * Hv, d_row_bits + l * Hv * stepq::kD,
                 d_row_off + l * Hv * stepq::kD, d_row_slot + l * Hv * stepq::kD};
     }
-    stepq::Shape shape() const {
-        return {cfg.n_key_heads, cfg.n_value_heads, cfg.n_layers,
-                cfg.gate_kind == STEPQ_GATE_CHANNEL ? 1 : 0,
-                cfg.gate_kind == STEPQ_GATE_CHANNEL ? 1 : 0, cfg.fit_iters};
-    }
 };
 
 namespace stepq {
@@ -92,12 +80,11 @@ stepq_status launch_decode(const stepq_plan *p, int layer, uint8_t *pool, int po
                            const int32_t *slots, int B, const float *q, const float *k,
                            const float *v, const float *beta, const float *gate, float *y,
                            cudaStream_t s);
-stepq_status launch_quantize(const stepq_plan *p, int layer, const float *states,
-                             size_t state_stride_b, const int32_t *slots, int B, uint8_t *pool,
-                             int pool_slots, cudaStream_t s);
+// layer = -1: every layer in one launch
+stepq_status launch_quantize(const stepq_plan *p, int layer, const float *states, const int32_t *slots, int B,
+                             uint8_t *pool, int pool_slots, cudaStream_t s);
 stepq_status launch_dequantize(const stepq_plan *p, int layer, const uint8_t *pool, int pool_slots,
-                               const int32_t *slots, int B, float *states, size_t state_stride_b,
-                               cudaStream_t s);
+                               const int32_t *slots, int B, float *states, cudaStream_t s);
 // prefill.cu (chunked FP32-state prefill)
 stepq_status launch_prefill(const stepq_config *cfg, const float *q, const float *k, const float *v,
                             const float *beta, const float *gate, int B, int T, float *states, float *y,
@@ -121,12 +108,10 @@ stepq_status launch_decode_heads_mode(const stepq_plan *p, int layer, uint8_t *p
                                       const int32_t *slots, int B, const float *q, const float *k,
                                       const float *v, const float *beta, const float *gate, float *y,
                                       float *delta, int mode, cudaStream_t s);
-stepq_status launch_quantize_heads(const stepq_plan *p, int layer, const float *states,
-                                   size_t stride_b, const int32_t *slots, int B, uint8_t *pool,
-                                   int pool_slots, cudaStream_t s);
-stepq_status launch_dequantize_heads(const stepq_plan *p, int layer, const uint8_t *pool,
-                                     int pool_slots, const int32_t *slots, int B, float *states,
-                                     size_t stride_b, cudaStream_t s);
+stepq_status launch_quantize_heads(const stepq_plan *p, int layer, const float *states, const int32_t *slots,
+                                   int B, uint8_t *pool, int pool_slots, cudaStream_t s);
+stepq_status launch_dequantize_heads(const stepq_plan *p, int layer, const uint8_t *pool, int pool_slots,
+                                     const int32_t *slots, int B, float *states, cudaStream_t s);
 // baselines.cu
 stepq_status launch_fp32_decode(const stepq_config *cfg, int layer, float *pool,
                                 const float *read_pool, int pool_slots, const int32_t *slots, int B,
@@ -165,6 +150,7 @@ stepq_status launch_validate_slots(const int32_t *slots, int B, int pool_slots,
 stepq_status launch_validate_slots_static(const int32_t *slots, int B, int pool_slots,
                                           int32_t *status, cudaStream_t s);
 stepq_status read_device_error(cudaStream_t s);
+int sm_count();                      // multiprocessors of the current device
 unsigned int *device_error_word();   // address of the current device's sticky error word
 // Test switch of the pipelined decode kernels (stepq_debug_stall): the bound of
 // every wait in SM cycles and an item whose copies never start (-1: none).

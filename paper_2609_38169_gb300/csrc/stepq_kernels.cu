@@ -2,9 +2,8 @@
 // (sm_103a), and the dispatch of the decode step: head units (GDN) run the
 // pipelined kernel of heads.cu, row units the one of rows.cu.
 //
-// One 256-thread CTA owns one (slot, value head) page: it stages the head
-// segment in shared memory with 128-bit loads, holds the tile in registers,
-// fits the dual-axis scales and writes the packed segment (App. C.3 steps 4-6).
+// A 256-thread CTA holds one (slot, value head) tile in registers, fits the
+// dual-axis scales and writes the packed segment (App. C.3 steps 4-6).
 //
 // Numerical contract (shared with the CPU oracle, which restates it in fp64):
 // the tile X is fp32; r_i = fp16(clamp(sqrt(m_i) * w_i^(-1/2), 2^-14, 65504));
@@ -336,94 +335,184 @@ __device__ __forceinline__ void copy16(uint4 *dst, const uint4 *src, int n16, in
 }
 
 // ---------------------------------------------------------- quantize / dequantize
-constexpr int kOffFit = (int)kMaxHeadBytes;                  // page [0, 33,280) | fit scratch | row offsets
-constexpr int kOffRoff = kOffFit + kFitBytes;                // int [128]
-constexpr int kSmemBytes = kOffRoff + 128 * 4;
-
 struct PoolArgs {
     uint8_t *pool;
     uint64_t stride;
     int pool_slots;
     const int32_t *slots;
     LayerTables tab;
-    Shape sh;
-    float *states;            // [B][..][Hv][128][128]
+    int heads, items;         // heads per batch entry (one layer's or all layers'); item = entry * heads + head
+    int fit_iters;
+    float *states;            // [B][..][heads][128][128]
     size_t state_stride_b;    // floats between consecutive batch entries
     unsigned int *err;
 };
 
+// Pack of dense states, persistent, two CTAs per SM. A state is 64 KB and its fit is
+// bound by instruction issue (about 8,000 warp instructions an item), so the loads
+// have to run under it: once an item's tile is in registers its shared-memory copy is
+// refilled with the next item's state (16-byte cp.async, swizzled as cgroup), and the
+// page leaves by a bulk store. One CTA per item with plain loads exposed their
+// latency (stalled on it 18% of the time at 24% occupancy): 4096 heads at 6 bits
+// took 143 us, 112 us now (47 us at the copy rate of HBM).
+constexpr int kQTile = 0;                                    // float [128][128], 16-byte groups swizzled
+constexpr int kQPage = kN * 4;
+constexpr int kQFit = kQPage + (int)kMaxHeadBytes;
+constexpr int kQRoff = kQFit + kFitBytes;                    // int [128]
+constexpr int kQSmem = kQRoff + 128 * 4;
+
 __global__ void __launch_bounds__(kThreads, 2) quantize_kernel(PoolArgs a) {
-    extern __shared__ __align__(16) uint8_t smem[];
+    extern __shared__ __align__(128) uint8_t smem[];
     const Lane L;
-    uint8_t *page = smem;
-    const FitSmem S(smem + kOffFit);
-    int *roff = (int *)(smem + kOffRoff);
-    const int Hv = a.sh.Hv;
-    const int b = blockIdx.x / Hv, h = blockIdx.x - b * Hv;
-    const int slot = a.slots[b];
-    if (slot < 0 || slot >= a.pool_slots) {
-        if (L.tid == 0) raise_error(a.err, STEPQ_ERR_SLOT_RANGE);
-        return;
+    float *tile = (float *)(smem + kQTile);
+    uint8_t *page = smem + kQPage;
+    const FitSmem S(smem + kQFit);
+    int *roff = (int *)(smem + kQRoff);
+    const int tid = L.tid;
+    const auto slot_of = [&](int item) { return item < a.items ? a.slots[item / a.heads] : -1; };
+    const auto ok = [&](int slot) { return slot >= 0 && slot < a.pool_slots; };
+    const auto start = [&](int item) {
+        const int b = item / a.heads, h = item - b * a.heads;
+        const float4 *X = (const float4 *)(a.states + (size_t)b * a.state_stride_b + (size_t)h * kN);
+#pragma unroll
+        for (int j = 0; j < 16; j++) {
+            const int e = tid + j * kThreads, row = e >> 5, f = e & 31;
+            cp_async16(&tile[row * 128 + 4 * cgroup(f >> 2, f & 3)], X + e);
+        }
+    };
+    // Row tables of an item's head: one row per thread of the first half.
+    int fbits = 0, froff = 0;
+    float fw2 = 0.f, fwis = 0.f;
+    const auto fetch = [&](int item) {
+        if (tid < 128) {
+            const int h = item % a.heads;
+            fbits = a.tab.row_bits[h * 128 + tid];
+            froff = (int)a.tab.row_off[h * 128 + tid];
+            fw2 = a.tab.w2[h * 128 + tid];
+            fwis = a.tab.wis[h * 128 + tid];
+        }
+    };
+    int slot = slot_of(blockIdx.x);
+    if (ok(slot)) {
+        start(blockIdx.x);
+        fetch(blockIdx.x);
     }
-    if (L.tid < 128) {
-        S.rbits[L.tid] = a.tab.row_bits[h * 128 + L.tid];
-        roff[L.tid] = (int)a.tab.row_off[h * 128 + L.tid];
-        S.w2[L.tid] = a.tab.w2[h * 128 + L.tid];
-        S.wis[L.tid] = a.tab.wis[h * 128 + L.tid];
+    for (int item = blockIdx.x; item < a.items; item += gridDim.x) {
+        const int next = item + gridDim.x, nslot = slot_of(next);
+        if (!ok(slot)) {                                      // uniform over the CTA
+            if (tid == 0) raise_error(a.err, STEPQ_ERR_SLOT_RANGE);
+            if (ok(nslot)) {
+                start(next);
+                fetch(next);
+            }
+            slot = nslot;
+            continue;
+        }
+        if (tid < 128) {
+            S.rbits[tid] = fbits;
+            roff[tid] = froff;
+            S.w2[tid] = fw2;
+            S.wis[tid] = fwis;
+        }
+        cp_async_wait_all();
+        __syncthreads();
+        uint64_t x[4][8];
+        float msum[4];
+#pragma unroll
+        for (int t = 0; t < 4; t++) {
+            float s = 0.f;
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const float4 f = *(const float4 *)&tile[L.row(t) * 128 + 4 * cgroup(L.cg, e)];
+                x[t][2 * e] = f2(f.x, f.y);
+                x[t][2 * e + 1] = f2(f.z, f.w);
+                s += fabsf(f.x) + fabsf(f.y) + fabsf(f.z) + fabsf(f.w);
+            }
+            msum[t] = row_allreduce(s);
+        }
+        if (tid == 0) bulk_wait_read_all();                   // the previous page has left
+        __syncthreads();
+        if (ok(nslot)) {
+            start(next);
+            fetch(next);
+        }
+        const bool clip = fit_scales(L, S, x, msum, 1, page, a.fit_iters);
+        pack_page(L, S, page, roff, x, clip);
+        fence_async_smem();
+        __syncthreads();
+        if (tid == 0) {
+            const int h = item % a.heads;
+            bulk_store(a.pool + (uint64_t)slot * a.stride + a.tab.head_off[h], page, a.tab.head_bytes[h]);
+            bulk_commit();
+        }
+        slot = nslot;
     }
-    uint64_t x[4][8];
-    float msum[4];
-    load_dense(L, a.states + (size_t)b * a.state_stride_b + (size_t)h * kN, x, msum);
-    __syncthreads();
-    const bool clip = fit_scales(L, S, x, msum, a.sh.unit_kind, page, a.sh.fit_iters);
-    pack_page(L, S, page, roff, x, clip);
-    __syncthreads();
-    uint8_t *gpage = a.pool + (uint64_t)slot * a.stride + a.tab.head_off[h];
-    copy16((uint4 *)gpage, (const uint4 *)page, (int)a.tab.head_bytes[h] >> 4, L.tid);
+    if (tid == 0) bulk_wait_all();
 }
 
-__global__ void __launch_bounds__(kThreads, 2) dequantize_kernel(PoolArgs a) {
-    extern __shared__ __align__(16) uint8_t smem[];
-    const Lane L;
-    uint8_t *page = smem;
-    int *rbits = (int *)(smem + kOffFit), *roff = (int *)(smem + kOffRoff);
-    const int Hv = a.sh.Hv;
-    const int b = blockIdx.x / Hv, h = blockIdx.x - b * Hv;
+// Unpack, one CTA per (slot, head) and bound by the 64 KB it writes. Warp w takes rows
+// 16w..16w+15 and lane l columns 4l..4l+3, so that a row's width is uniform over the
+// warp, its codes are read straight from the page and its 512 bytes leave as one
+// store instruction. (Staging the page in shared memory with 16 columns of a row per
+// thread wrote in 16-byte pieces 64 bytes apart and waited for the staging: 88 us for
+// 4096 heads at 6 bits, 54 us now; 47 us at the copy rate of HBM.)
+__global__ void __launch_bounds__(kThreads, 4) dequantize_kernel(PoolArgs a) {
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    const int b = blockIdx.x / a.heads, h = blockIdx.x - b * a.heads;
     const int slot = a.slots[b];
     if (slot < 0 || slot >= a.pool_slots) {
-        if (L.tid == 0) raise_error(a.err, STEPQ_ERR_SLOT_RANGE);
+        if (threadIdx.x == 0) raise_error(a.err, STEPQ_ERR_SLOT_RANGE);
         return;
     }
-    const uint8_t *gpage = a.pool + (uint64_t)slot * a.stride + a.tab.head_off[h];
-    copy16((uint4 *)page, (const uint4 *)gpage, (int)a.tab.head_bytes[h] >> 4, L.tid);
-    if (L.tid < 128) {
-        rbits[L.tid] = a.tab.row_bits[h * 128 + L.tid];
-        roff[L.tid] = (int)a.tab.row_off[h * 128 + L.tid];
-    }
-    __syncthreads();
-    const int has_scales = a.tab.head_bits[h] != kPivot;
-    const uint16_t *page_r = (const uint16_t *)page;
-    const uint16_t *page_c = (const uint16_t *)(page + 256);
+    const uint8_t *page = a.pool + (uint64_t)slot * a.stride + a.tab.head_off[h];
     float *out = a.states + (size_t)b * a.state_stride_b + (size_t)h * kN;
+    // Lanes 0..15: width, payload offset and r_i zs_i (exact) of the warp's rows.
+    int tbits = 0, toff = 0;
+    float trz = 0.f;
+    if (l < 16) {
+        const int i = 16 * w + l;
+        tbits = a.tab.row_bits[h * 128 + i];
+        toff = (int)a.tab.row_off[h * 128 + i];
+        const float r = f16_val(((const uint16_t *)page)[i]);
+        if (tbits != kPivot) trz = r * (float)(1 << (8 - tbits));
+    }
+    const uint2 c4 = ((const uint2 *)(page + 256))[l];
+    const uint64_t c01 = f2(f16_val((uint16_t)(c4.x & 0xFFFFu)), f16_val((uint16_t)(c4.x >> 16)));
+    const uint64_t c23 = f2(f16_val((uint16_t)(c4.y & 0xFFFFu)), f16_val((uint16_t)(c4.y >> 16)));
 #pragma unroll
-    for (int t = 0; t < 4; t++) {
-        const int i = L.row(t);
-        const int bits = rbits[i];
-        float vals[16];
-        load_row16(page + roff[i], bits, L.cg, vals);
-        if (bits != kPivot) {
-            const float r = f16_val(page_r[i]);
-            const float zs = a.sh.unit_kind ? (float)(1 << (8 - bits)) : 1.f;
+    for (int r0 = 0; r0 < 16; r0 += 8) {
+        // The words that hold the lane's 4b bits of eight rows (its first byte is
+        // l b / 2; an FP16 row has two whole words). The second word is read only
+        // where the lane's bits reach it, so no read passes the row.
+        uint32_t w0[8], w1[8];
 #pragma unroll
-            for (int j = 0; j < 16; j++) {
-                const float rc = r * (has_scales ? f16_val(page_c[L.col0() + j]) : 1.f);
-                vals[j] = __fmul_rn(rc, zs * vals[j]);       // one rounding of r c z
-            }
+        for (int u = 0; u < 8; u++) {
+            const int bits = __shfl_sync(0xffffffffu, tbits, r0 + u), off = __shfl_sync(0xffffffffu, toff, r0 + u);
+            const int at = (l * bits) >> 1;
+            const uint32_t *p = (const uint32_t *)(page + off + (at & ~3));
+            w0[u] = p[0];
+            w1[u] = 8 * (at & 3) + 4 * bits > 32 ? p[1] : 0u;
         }
-        float4 *dst = (float4 *)(out + i * 128 + L.col0());
 #pragma unroll
-        for (int e = 0; e < 4; e++)
-            dst[e] = make_float4(vals[4 * e], vals[4 * e + 1], vals[4 * e + 2], vals[4 * e + 3]);
+        for (int u = 0; u < 8; u++) {
+            const int bits = __shfl_sync(0xffffffffu, tbits, r0 + u);
+            const float rz = __shfl_sync(0xffffffffu, trz, r0 + u);
+            float4 v;
+            if (bits == kPivot) {
+                v = make_float4(f16_val((uint16_t)(w0[u] & 0xFFFFu)), f16_val((uint16_t)(w0[u] >> 16)),
+                                f16_val((uint16_t)(w1[u] & 0xFFFFu)), f16_val((uint16_t)(w1[u] >> 16)));
+            } else {
+                const uint32_t s = __funnelshift_r(w0[u], w1[u], 8 * (((l * bits) >> 1) & 3)), m = (1u << bits) - 1u;
+                const uint64_t off = f2s(-(kMagic + (float)(1 << (bits - 1)))), rz2 = f2s(rz);
+                // q is exact, r c zs is exact (22 bits), their product rounds once
+                const uint64_t q01 = fadd2(u2pair(and_or(s, m, kMagicBits), and_or(s >> bits, m, kMagicBits)), off);
+                const uint64_t q23 =
+                    fadd2(u2pair(and_or(s >> (2 * bits), m, kMagicBits), and_or(s >> (3 * bits), m, kMagicBits)), off);
+                const uint64_t v01 = fmul2(fmul2(rz2, c01), q01), v23 = fmul2(fmul2(rz2, c23), q23);
+                v = make_float4(f2lo(v01), f2hi(v01), f2lo(v23), f2hi(v23));
+            }
+            *(float4 *)(out + (16 * w + r0 + u) * 128 + 4 * l) = v;
+        }
     }
 }
 
@@ -574,7 +663,7 @@ constexpr int kRpAcc = (kRpFit + kFitBytes + 15) / 16 * 16;  // double [128][5]
 constexpr int kRpSmem = kRpAcc + 128 * 5 * 8;
 
 __global__ void __launch_bounds__(kThreads, 2) replay_kernel(ReplayArgs a) {
-    extern __shared__ __align__(16) uint8_t smem[];
+    extern __shared__ __align__(128) uint8_t smem[];
     const Lane L;
     const FitSmem S(smem + kRpFit);
     float *tile = (float *)(smem + kRpTile), *red = (float *)(smem + kRpRed), *vs = (float *)(smem + kRpV);
@@ -704,9 +793,7 @@ static stepq_status prepare(int dev) {
     if (dev < 0 || dev >= 64) return STEPQ_ERR_CUDA;
     if (!g_attr_set[dev]) {
         if (cudaFuncSetAttribute(quantize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kSmemBytes) != cudaSuccess ||
-            cudaFuncSetAttribute(dequantize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kSmemBytes) != cudaSuccess ||
+                                 kQSmem) != cudaSuccess ||
             cudaFuncSetAttribute(replay_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  kRpSmem) != cudaSuccess)
             return STEPQ_ERR_CUDA;
@@ -728,29 +815,33 @@ stepq_status launch_decode(const stepq_plan *p, int layer, uint8_t *pool, int po
     return launch_decode_rows(p, layer, pool, pool_slots, slots, B, q, k, v, beta, gate, y, s);
 }
 
-stepq_status launch_quantize(const stepq_plan *p, int layer, const float *states,
-                             size_t state_stride_b, const int32_t *slots, int B, uint8_t *pool,
-                             int pool_slots, cudaStream_t s) {
+// layer >= 0: one layer's heads; layer = -1: all layers' in one launch (their tables,
+// and their states in a batch entry, follow each other).
+static PoolArgs pool_args(const stepq_plan *p, int layer, const float *states, const int32_t *slots, int B,
+                          uint8_t *pool, int pool_slots) {
+    const int heads = p->cfg.n_value_heads * (layer < 0 ? p->cfg.n_layers : 1);
+    return {pool, p->slot_stride, pool_slots, slots, p->layer(layer < 0 ? 0 : layer), heads, B * heads,
+            p->cfg.fit_iters, (float *)states, (size_t)heads * kN, device_error_word()};
+}
+
+stepq_status launch_quantize(const stepq_plan *p, int layer, const float *states, const int32_t *slots, int B,
+                             uint8_t *pool, int pool_slots, cudaStream_t s) {
     if (p->cfg.gate_kind == STEPQ_GATE_SCALAR)
-        return launch_quantize_heads(p, layer, states, state_stride_b, slots, B, pool, pool_slots, s);
+        return launch_quantize_heads(p, layer, states, slots, B, pool, pool_slots, s);
     stepq_status st = prepare(p->device);
     if (st != STEPQ_OK) return st;
-    PoolArgs a{pool, p->slot_stride, pool_slots, slots, p->layer(layer), p->shape(),
-               (float *)states, state_stride_b, device_error_word()};
-    quantize_kernel<<<(unsigned)B * p->cfg.n_value_heads, kThreads, kSmemBytes, s>>>(a);
+    const PoolArgs a = pool_args(p, layer, states, slots, B, pool, pool_slots);
+    const int grid = 2 * sm_count();
+    quantize_kernel<<<grid < a.items ? grid : a.items, kThreads, kQSmem, s>>>(a);
     return launched();
 }
 
 stepq_status launch_dequantize(const stepq_plan *p, int layer, const uint8_t *pool, int pool_slots,
-                               const int32_t *slots, int B, float *states, size_t state_stride_b,
-                               cudaStream_t s) {
+                               const int32_t *slots, int B, float *states, cudaStream_t s) {
     if (p->cfg.gate_kind == STEPQ_GATE_SCALAR)
-        return launch_dequantize_heads(p, layer, pool, pool_slots, slots, B, states, state_stride_b, s);
-    stepq_status st = prepare(p->device);
-    if (st != STEPQ_OK) return st;
-    PoolArgs a{(uint8_t *)pool, p->slot_stride, pool_slots, slots, p->layer(layer), p->shape(),
-               states, state_stride_b, device_error_word()};
-    dequantize_kernel<<<(unsigned)B * p->cfg.n_value_heads, kThreads, kSmemBytes, s>>>(a);
+        return launch_dequantize_heads(p, layer, pool, pool_slots, slots, B, states, s);
+    const PoolArgs a = pool_args(p, layer, states, slots, B, (uint8_t *)pool, pool_slots);
+    dequantize_kernel<<<a.items, kThreads, 0, s>>>(a);
     return launched();
 }
 
