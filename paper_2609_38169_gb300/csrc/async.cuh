@@ -100,6 +100,15 @@ __device__ __forceinline__ void fence_async_smem() {
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+// ---- programmatic dependent launch ----
+// A kernel launched with launch_overlapped() may start before the stream's previous
+// kernel has ended: nothing that depends on earlier work is read, and nothing is
+// written, before griddep_wait() (which returns once that work is complete and
+// visible). griddep_launch() lets the next such kernel start as soon as every CTA of
+// this one has called it or ended.
+__device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void griddep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // ---- packed fp32 pairs (sm_100+) ----
 __device__ __forceinline__ uint64_t f2(float a, float b) {
     uint64_t d;

@@ -47,6 +47,17 @@ int sm_count() {
     return v > 0 ? v : 1;
 }
 
+stepq_status SmemOptIn::operator()(const void *kernel, int bytes) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return STEPQ_ERR_CUDA;
+    const uint64_t bit = 1ull << dev;
+    if (done.load(std::memory_order_acquire) & bit) return STEPQ_OK;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess)
+        return STEPQ_ERR_CUDA;
+    done.fetch_or(bit, std::memory_order_release);
+    return STEPQ_OK;
+}
+
 // The pipelined kernels' wait bound and withheld item (test support). Plain
 // process-wide values: stepq_debug_stall is documented as not thread-safe.
 static long long g_wait_cycles = pipe::kWaitCycles;

@@ -60,6 +60,8 @@ __global__ void __launch_bounds__(kThreads, 1) decode_kernel(DecodeArgs a) {
         mbar_init_fence();
     }
     __syncthreads();
+    griddep_wait();
+    griddep_launch();
     const int grp = a.Hv / a.Hk;
     const auto page_of = [&](int h, int slot) {
         return a.pool + (uint64_t)slot * a.slot_bytes + a.layer_off + (uint64_t)h * kPage;
@@ -186,22 +188,18 @@ stepq_status launch_fp32_decode(const stepq_config *cfg, int layer, float *pool,
     a.q = q; a.k = k; a.v = v; a.beta = beta; a.gate = gate; a.y = y;
     a.err = device_error_word();
     a.stall = stall_knob();
-    int dev = 0, sms = 1, max_smem = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    int stages = (max_smem - fk::kOffStages) / fk::kStage;
-    stages = stages < 2 ? 2 : (stages > 3 ? 3 : stages);
+    constexpr int stages = (kSmemMax - fk::kOffStages) / fk::kStage < 3 ? (kSmemMax - fk::kOffStages) / fk::kStage : 3;
+    static_assert(stages >= 2, "the page pipeline needs two stages");
     a.n_stages = stages;
     const int smem = fk::kOffStages + stages * fk::kStage;
-    const void *fn = read_pool ? (const void *)fk::decode_kernel<true> : (const void *)fk::decode_kernel<false>;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-        return STEPQ_ERR_CUDA;
-    int grid = sms > 0 ? sms : 1;
+    int grid = sm_count();
     if (grid > a.items) grid = a.items;
-    if (read_pool) fk::decode_kernel<true><<<grid, kThreads, smem, s>>>(a);
-    else fk::decode_kernel<false><<<grid, kThreads, smem, s>>>(a);
-    return cudaGetLastError() == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
+    static SmemOptIn opt[2];
+    const auto launch = [&](auto kernel) {
+        const stepq_status st = opt[read_pool != nullptr]((const void *)kernel, smem);
+        return st == STEPQ_OK ? launch_overlapped(kernel, grid, kThreads, smem, s, a) : st;
+    };
+    return read_pool ? launch(fk::decode_kernel<true>) : launch(fk::decode_kernel<false>);
 }
 
 }  // namespace stepq

@@ -625,6 +625,8 @@ __global__ void __launch_bounds__(kThreads, 2) decode_heads_kernel(DecodeArgs a)
         mbar_init_fence();
     }
     __syncthreads();
+    griddep_wait();
+    griddep_launch();
     const pipe::Shape p{a.items, a.nb, a.n_stages, a.slots, a.pool_slots, a.err, a.stall.wait_cycles,
                         a.stall.withhold_item};
     pipe::run(
@@ -683,6 +685,8 @@ __global__ void __launch_bounds__(kThreads, 2) quantize_heads_kernel(PoolArgs a)
     extern __shared__ __align__(128) uint8_t smem[];
     const T t;
     const Smem S(smem);
+    griddep_wait();
+    griddep_launch();
     float *tile = (float *)(smem + kOffQTile), *w2 = (float *)(smem + kOffQVec), *wis = w2 + 128;
     uint8_t *page = smem + kOffQPage;
     const auto slot_of = [&](int item) { return item < a.items ? a.slots[item / a.heads] : -1; };
@@ -787,6 +791,8 @@ __global__ void __launch_bounds__(kThreads, 3) dequantize_heads_kernel(PoolArgs 
     extern __shared__ __align__(128) uint8_t smem[];
     const T t;
     const int b = blockIdx.x / a.heads, h = blockIdx.x - b * a.heads;
+    griddep_wait();
+    griddep_launch();
     const int slot = a.slots[b];
     if (slot < 0 || slot >= a.pool_slots) {
         if (t.tid == 0) raise_error(a.err, STEPQ_ERR_SLOT_RANGE);
@@ -813,12 +819,6 @@ __global__ void __launch_bounds__(kThreads, 3) dequantize_heads_kernel(PoolArgs 
 }  // namespace hk
 
 // ------------------------------------------------------------------ launchers
-static stepq_status set_attr(const void *fn, int bytes) {
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) == cudaSuccess
-               ? STEPQ_OK
-               : STEPQ_ERR_CUDA;
-}
-
 stepq_status launch_decode_heads(const stepq_plan *p, int layer, uint8_t *pool, int pool_slots,
                                  const int32_t *slots, int B, const float *q, const float *k,
                                  const float *v, const float *beta, const float *gate, float *y,
@@ -858,16 +858,16 @@ stepq_status launch_decode_heads_mode(const stepq_plan *p, int layer, uint8_t *p
     a.n_stages = stages;
     a.fit_iters = p->cfg.fit_iters;
     const int smem = hk::kOffStages + stages * (int)a.stage_bytes;
-    const void *fn = mode == hk::kReadout     ? (const void *)hk::decode_heads_kernel<hk::kReadout>
-                     : mode == hk::kWriteback ? (const void *)hk::decode_heads_kernel<hk::kWriteback>
-                                              : (const void *)hk::decode_heads_kernel<hk::kFused>;
-    if (set_attr(fn, smem) != STEPQ_OK) return STEPQ_ERR_CUDA;
     int grid = 2 * sm_count();
     if (grid > a.items) grid = a.items;
-    if (mode == hk::kReadout) hk::decode_heads_kernel<hk::kReadout><<<grid, kThreads, smem, s>>>(a);
-    else if (mode == hk::kWriteback) hk::decode_heads_kernel<hk::kWriteback><<<grid, kThreads, smem, s>>>(a);
-    else hk::decode_heads_kernel<hk::kFused><<<grid, kThreads, smem, s>>>(a);
-    return cudaGetLastError() == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
+    static SmemOptIn opt[3];
+    const auto launch = [&](auto kernel) {
+        const stepq_status st = opt[mode]((const void *)kernel, kSmemMax);
+        return st == STEPQ_OK ? launch_overlapped(kernel, grid, kThreads, smem, s, a) : st;
+    };
+    if (mode == hk::kReadout) return launch(hk::decode_heads_kernel<hk::kReadout>);
+    if (mode == hk::kWriteback) return launch(hk::decode_heads_kernel<hk::kWriteback>);
+    return launch(hk::decode_heads_kernel<hk::kFused>);
 }
 
 static hk::PoolArgs pool_args(const stepq_plan *p, int layer, const float *states, const int32_t *slots, int B,
@@ -879,19 +879,21 @@ static hk::PoolArgs pool_args(const stepq_plan *p, int layer, const float *state
 
 stepq_status launch_quantize_heads(const stepq_plan *p, int layer, const float *states, const int32_t *slots,
                                    int B, uint8_t *pool, int pool_slots, cudaStream_t s) {
-    if (set_attr((const void *)hk::quantize_heads_kernel, hk::kPackSmem) != STEPQ_OK) return STEPQ_ERR_CUDA;
+    static SmemOptIn opt;
+    const stepq_status st = opt((const void *)hk::quantize_heads_kernel, hk::kPackSmem);
+    if (st != STEPQ_OK) return st;
     const hk::PoolArgs a = pool_args(p, layer, states, slots, B, pool, pool_slots);
     const int grid = 2 * sm_count();
-    hk::quantize_heads_kernel<<<grid < a.items ? grid : a.items, kThreads, hk::kPackSmem, s>>>(a);
-    return cudaGetLastError() == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
+    return launch_overlapped(hk::quantize_heads_kernel, grid < a.items ? grid : a.items, kThreads, hk::kPackSmem, s, a);
 }
 
 stepq_status launch_dequantize_heads(const stepq_plan *p, int layer, const uint8_t *pool, int pool_slots,
                                      const int32_t *slots, int B, float *states, cudaStream_t s) {
-    if (set_attr((const void *)hk::dequantize_heads_kernel, hk::kUnpackSmem) != STEPQ_OK) return STEPQ_ERR_CUDA;
+    static SmemOptIn opt;
+    const stepq_status st = opt((const void *)hk::dequantize_heads_kernel, hk::kUnpackSmem);
+    if (st != STEPQ_OK) return st;
     const hk::PoolArgs a = pool_args(p, layer, states, slots, B, (uint8_t *)pool, pool_slots);
-    hk::dequantize_heads_kernel<<<a.items, kThreads, hk::kUnpackSmem, s>>>(a);
-    return cudaGetLastError() == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
+    return launch_overlapped(hk::dequantize_heads_kernel, a.items, kThreads, hk::kUnpackSmem, s, a);
 }
 
 }  // namespace stepq

@@ -323,6 +323,8 @@ __global__ void __launch_bounds__(kThreads, 2) decode_kernel(DecodeArgs a, int b
         mbar_init_fence();
     }
     __syncthreads();
+    griddep_wait();
+    griddep_launch();
     const int grp = a.Hv / a.Hk;
     const auto page_of = [&](int h, int slot) {
         return a.pool + (uint64_t)slot * a.slot_bytes + a.layer_off + (uint64_t)h * a.head_bytes;
@@ -394,16 +396,12 @@ stepq_status launch_intb_decode(const stepq_config *cfg, int bits, int layer, ui
     stages = stages < 2 ? 2 : (stages > 4 ? 4 : stages);
     a.n_stages = stages;
     const int smem = ib::kOffStages + stages * (int)a.stage_bytes;
-    if (cudaFuncSetAttribute((const void *)ib::decode_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             smem) != cudaSuccess)
-        return STEPQ_ERR_CUDA;
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int grid = 2 * (sms > 0 ? sms : 1);
+    static SmemOptIn opt;
+    const stepq_status st = opt((const void *)ib::decode_kernel, kSmemMax);
+    if (st != STEPQ_OK) return st;
+    int grid = 2 * sm_count();
     if (grid > a.items) grid = a.items;
-    ib::decode_kernel<<<grid, kThreads, smem, s>>>(a, bits);
-    return cudaGetLastError() == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
+    return launch_overlapped(ib::decode_kernel, grid, kThreads, smem, s, a, bits);
 }
 
 }  // namespace stepq

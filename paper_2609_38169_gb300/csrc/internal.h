@@ -1,6 +1,7 @@
 // Internal definitions shared by the library's translation units (not part of the ABI).
 #pragma once
 
+#include <atomic>
 #include <cstddef>
 #include <cstdint>
 #include <vector>
@@ -151,6 +152,36 @@ stepq_status launch_validate_slots_static(const int32_t *slots, int B, int pool_
                                           int32_t *status, cudaStream_t s);
 stepq_status read_device_error(cudaStream_t s);
 int sm_count();                      // multiprocessors of the current device
+
+// Launch of a kernel that may overlap the end of the stream's previous kernel: its
+// CTAs take their places, and run up to griddep_wait(), as that kernel's CTAs leave.
+// A decode launch spends about 3 us before its first page arrives (placing the
+// CTAs, tables, barriers) which then no longer follow the previous layer's end.
+// Captures into graphs like a plain launch.
+template <class Args, class... Rest>
+inline stepq_status launch_overlapped(void (*kernel)(Args, Rest...), int grid, int block, int smem, cudaStream_t s,
+                                      const Args &a, Rest... rest) {
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)block);
+    c.dynamicSmemBytes = (size_t)smem;
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, a, rest...) == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
+}
+
+constexpr int kSmemMax = 227 * 1024;   // dynamic shared memory one CTA can have
+
+// Allows `kernel` the dynamic shared memory a launch may take, once per device (the
+// flags are bit sets over devices; setting it twice is harmless).
+struct SmemOptIn {
+    std::atomic<uint64_t> done{0};
+    stepq_status operator()(const void *kernel, int bytes);
+};
 unsigned int *device_error_word();   // address of the current device's sticky error word
 // Test switch of the pipelined decode kernels (stepq_debug_stall): the bound of
 // every wait in SM cycles and an item whose copies never start (-1: none).

@@ -132,6 +132,8 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(Args a) {
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
+    griddep_wait();
+    griddep_launch();
     const uint32_t tm = *tbase;                            // lane 0, first column
     const uint32_t tl = tm + ((uint32_t)(32 * quad) << 16);   // this warp's lanes
     uint32_t parity = 0;
@@ -429,16 +431,12 @@ stepq_status launch_prefill(const stepq_config *cfg, const float *q, const float
     a.gate_per_row = cfg->gate_kind == STEPQ_GATE_CHANNEL;
     a.items = B * a.Hv;
     a.err = device_error_word();
-    if (cudaFuncSetAttribute((const void *)pf::prefill_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             pf::kSmem) != cudaSuccess)
-        return STEPQ_ERR_CUDA;
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int grid = sms > 0 ? sms : 1;
+    static SmemOptIn opt;
+    const stepq_status st = opt((const void *)pf::prefill_kernel, pf::kSmem);
+    if (st != STEPQ_OK) return st;
+    int grid = sm_count();
     if (grid > a.items) grid = a.items;
-    pf::prefill_kernel<<<grid, kThreads, pf::kSmem, s>>>(a);
-    return cudaGetLastError() == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
+    return launch_overlapped(pf::prefill_kernel, grid, kThreads, pf::kSmem, s, a);
 }
 
 }  // namespace stepq

@@ -621,6 +621,8 @@ __global__ void __launch_bounds__(kThreads, 2) decode_rows_kernel(DecodeArgs a) 
         mbar_init_fence();
     }
     __syncthreads();
+    griddep_wait();
+    griddep_launch();
     const pipe::Shape p{a.items, a.nb, a.n_stages, a.slots, a.pool_slots, a.err, a.stall.wait_cycles,
                         a.stall.withhold_item};
     pipe::run(
@@ -681,20 +683,16 @@ stepq_status launch_decode_rows_mode(const stepq_plan *p, int layer, uint8_t *po
     a.n_stages = stages;
     a.fit_iters = p->cfg.fit_iters;
     const int smem = rk::kOffStages + stages * (int)a.stage_bytes;
-    const void *fn = mode == rk::kReadout     ? (const void *)rk::decode_rows_kernel<rk::kReadout>
-                     : mode == rk::kWriteback ? (const void *)rk::decode_rows_kernel<rk::kWriteback>
-                                              : (const void *)rk::decode_rows_kernel<rk::kFused>;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
-        return STEPQ_ERR_CUDA;
-    int dev = 0, sms = 1;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    int grid = 2 * (sms > 0 ? sms : 1);
+    int grid = 2 * sm_count();
     if (grid > a.items) grid = a.items;
-    if (mode == rk::kReadout) rk::decode_rows_kernel<rk::kReadout><<<grid, kThreads, smem, s>>>(a);
-    else if (mode == rk::kWriteback) rk::decode_rows_kernel<rk::kWriteback><<<grid, kThreads, smem, s>>>(a);
-    else rk::decode_rows_kernel<rk::kFused><<<grid, kThreads, smem, s>>>(a);
-    return cudaGetLastError() == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
+    static SmemOptIn opt[3];
+    const auto launch = [&](auto kernel) {
+        const stepq_status st = opt[mode]((const void *)kernel, kSmemMax);
+        return st == STEPQ_OK ? launch_overlapped(kernel, grid, kThreads, smem, s, a) : st;
+    };
+    if (mode == rk::kReadout) return launch(rk::decode_rows_kernel<rk::kReadout>);
+    if (mode == rk::kWriteback) return launch(rk::decode_rows_kernel<rk::kWriteback>);
+    return launch(rk::decode_rows_kernel<rk::kFused>);
 }
 
 }  // namespace stepq

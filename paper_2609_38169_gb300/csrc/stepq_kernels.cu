@@ -13,9 +13,6 @@
 // c is fitted from the clip-free start
 // max_i fp32(fp32(|X_ij| rho_i) / qmax_i) by `fit_iters` fixed-code
 // least-squares updates.
-#include <atomic>
-#include <cstdio>
-
 #include "async.cuh"
 #include "device.cuh"
 #include "internal.h"
@@ -369,6 +366,8 @@ __global__ void __launch_bounds__(kThreads, 2) quantize_kernel(PoolArgs a) {
     const FitSmem S(smem + kQFit);
     int *roff = (int *)(smem + kQRoff);
     const int tid = L.tid;
+    griddep_wait();
+    griddep_launch();
     const auto slot_of = [&](int item) { return item < a.items ? a.slots[item / a.heads] : -1; };
     const auto ok = [&](int slot) { return slot >= 0 && slot < a.pool_slots; };
     const auto start = [&](int item) {
@@ -459,6 +458,8 @@ __global__ void __launch_bounds__(kThreads, 2) quantize_kernel(PoolArgs a) {
 __global__ void __launch_bounds__(kThreads, 4) dequantize_kernel(PoolArgs a) {
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     const int b = blockIdx.x / a.heads, h = blockIdx.x - b * a.heads;
+    griddep_wait();
+    griddep_launch();
     const int slot = a.slots[b];
     if (slot < 0 || slot >= a.pool_slots) {
         if (threadIdx.x == 0) raise_error(a.err, STEPQ_ERR_SLOT_RANGE);
@@ -786,22 +787,6 @@ __global__ void __launch_bounds__(kThreads, 2) replay_kernel(ReplayArgs a) {
 }
 
 // ------------------------------------------------------------------ launchers
-static std::atomic<bool> g_attr_set[64];   // per device; setting the attributes twice is harmless
-
-static stepq_status prepare(int dev) {
-    if (dev < 0) cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 64) return STEPQ_ERR_CUDA;
-    if (!g_attr_set[dev]) {
-        if (cudaFuncSetAttribute(quantize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kQSmem) != cudaSuccess ||
-            cudaFuncSetAttribute(replay_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kRpSmem) != cudaSuccess)
-            return STEPQ_ERR_CUDA;
-        g_attr_set[dev] = true;
-    }
-    return STEPQ_OK;
-}
-
 static stepq_status launched() {
     return cudaGetLastError() == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
 }
@@ -828,12 +813,12 @@ stepq_status launch_quantize(const stepq_plan *p, int layer, const float *states
                              uint8_t *pool, int pool_slots, cudaStream_t s) {
     if (p->cfg.gate_kind == STEPQ_GATE_SCALAR)
         return launch_quantize_heads(p, layer, states, slots, B, pool, pool_slots, s);
-    stepq_status st = prepare(p->device);
+    static SmemOptIn opt;
+    const stepq_status st = opt((const void *)quantize_kernel, kQSmem);
     if (st != STEPQ_OK) return st;
     const PoolArgs a = pool_args(p, layer, states, slots, B, pool, pool_slots);
     const int grid = 2 * sm_count();
-    quantize_kernel<<<grid < a.items ? grid : a.items, kThreads, kQSmem, s>>>(a);
-    return launched();
+    return launch_overlapped(quantize_kernel, grid < a.items ? grid : a.items, kThreads, kQSmem, s, a);
 }
 
 stepq_status launch_dequantize(const stepq_plan *p, int layer, const uint8_t *pool, int pool_slots,
@@ -841,8 +826,7 @@ stepq_status launch_dequantize(const stepq_plan *p, int layer, const uint8_t *po
     if (p->cfg.gate_kind == STEPQ_GATE_SCALAR)
         return launch_dequantize_heads(p, layer, pool, pool_slots, slots, B, states, s);
     const PoolArgs a = pool_args(p, layer, states, slots, B, (uint8_t *)pool, pool_slots);
-    dequantize_kernel<<<a.items, kThreads, 0, s>>>(a);
-    return launched();
+    return launch_overlapped(dequantize_kernel, a.items, kThreads, 0, s, a);
 }
 
 static FitCands fit_cands(const stepq_config *cfg) {
@@ -874,7 +858,8 @@ stepq_status launch_calib_distortion(const stepq_config *cfg, int layer, const f
 stepq_status launch_calib_replay(const stepq_config *cfg, int n, int T, int every, const float *k,
                                  const float *v, const float *beta, const float *gate, const float *w,
                                  const uint8_t *pivot_rows, double *acc, cudaStream_t s) {
-    stepq_status st = prepare(-1);
+    static SmemOptIn opt;
+    const stepq_status st = opt((const void *)replay_kernel, kRpSmem);
     if (st != STEPQ_OK) return st;
     const bool rows = cfg->gate_kind == STEPQ_GATE_CHANNEL;
     ReplayArgs a{k, v, beta, gate, w, rows ? pivot_rows : nullptr, acc, n, T, cfg->n_key_heads,
