@@ -72,19 +72,49 @@ def _dev_ptr(t, dtype=None):
     """Device pointer of a contiguous CUDA tensor (None passes through)."""
     if t is None:
         return None
+    if t.is_cuda and t.is_contiguous() and (dtype is None or t.dtype is dtype):
+        return t.data_ptr()
     if not t.is_cuda:
         raise ValueError("expected a CUDA tensor")
     if not t.is_contiguous():
         raise ValueError("expected a contiguous tensor")
-    if dtype is not None and t.dtype != dtype:
-        raise ValueError(f"expected {dtype}, got {t.dtype}")
-    return t.data_ptr()
+    raise ValueError(f"expected {dtype}, got {t.dtype}")
+
+
+class _Torch:
+    """What a call needs of torch, looked up once (torch is imported with the first
+    device call; the host-side plan functions work without it)."""
+    f32 = f64 = i32 = u8 = None
+    _raw = None
+
+    @classmethod
+    def load(cls):
+        import torch
+        cls.f64, cls.i32, cls.u8 = torch.float64, torch.int32, torch.uint8
+        cls.f32 = torch.float32
+
+    @classmethod
+    def stream(cls):
+        """Handle of the current device's current stream, without the Stream object
+        around it where torch offers that (0.2 us a call instead of 3.1)."""
+        if cls._raw is None:
+            import torch
+            handle = torch.cuda.current_stream().cuda_stream        # initialises CUDA
+            get, device = (getattr(torch._C, n, None) for n in ("_cuda_getCurrentRawStream", "_cuda_getDevice"))
+            if get is None or device is None:
+                return handle
+            cls._raw = staticmethod(lambda: get(device()))
+        return cls._raw()
+
+
+def _f32():
+    if _Torch.f32 is None:
+        _Torch.load()
+    return _Torch.f32
 
 
 def _stream(stream):
-    import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    return _Torch.stream() if stream is None else stream.cuda_stream
 
 
 def version() -> str:
@@ -185,22 +215,22 @@ def alloc_pool(plan: Plan, pool_slots: int, device="cuda"):
 
 
 def stepq_quantize_pool(plan: Plan, layer: int, states, slots, pool, pool_slots=None, stream=None):
-    import torch
+    f = _f32()
     B = slots.numel()
-    check(_lib.lib().stepq_quantize_pool(plan.handle, layer, _dev_ptr(states, torch.float32),
-                                         _dev_ptr(slots, torch.int32), B, _dev_ptr(pool),
+    check(_lib.lib().stepq_quantize_pool(plan.handle, layer, _dev_ptr(states, f),
+                                         _dev_ptr(slots, _Torch.i32), B, _dev_ptr(pool),
                                          _pool_slots(pool, plan.slot_stride, pool_slots),
                                          _stream(stream)), "stepq_quantize_pool")
 
 
 def stepq_dequantize_pool(plan: Plan, layer: int, pool, slots, states_out, pool_slots=None,
                           stream=None):
-    import torch
+    f = _f32()
     B = slots.numel()
     check(_lib.lib().stepq_dequantize_pool(plan.handle, layer, _dev_ptr(pool),
                                            _pool_slots(pool, plan.slot_stride, pool_slots),
-                                           _dev_ptr(slots, torch.int32), B,
-                                           _dev_ptr(states_out, torch.float32), _stream(stream)),
+                                           _dev_ptr(slots, _Torch.i32), B,
+                                           _dev_ptr(states_out, f), _stream(stream)),
           "stepq_dequantize_pool")
 
 
@@ -210,33 +240,32 @@ def stepq_temporal_slot_bytes(plan: Plan) -> int:
 
 def stepq_temporal_quantize_pool(plan: Plan, layer: int, states, slots, pool, pool_slots=None,
                                  stream=None):
-    import torch
+    f = _f32()
     stride = stepq_temporal_slot_bytes(plan)
-    check(_lib.lib().stepq_temporal_quantize_pool(plan.handle, layer, _dev_ptr(states, torch.float32),
-                                                  _dev_ptr(slots, torch.int32), slots.numel(),
+    check(_lib.lib().stepq_temporal_quantize_pool(plan.handle, layer, _dev_ptr(states, f),
+                                                  _dev_ptr(slots, _Torch.i32), slots.numel(),
                                                   _dev_ptr(pool), _pool_slots(pool, stride, pool_slots),
                                                   _stream(stream)), "stepq_temporal_quantize_pool")
 
 
 def stepq_temporal_dequantize_pool(plan: Plan, layer: int, pool, slots, states_out, pool_slots=None,
                                    stream=None):
-    import torch
+    f = _f32()
     stride = stepq_temporal_slot_bytes(plan)
     check(_lib.lib().stepq_temporal_dequantize_pool(plan.handle, layer, _dev_ptr(pool),
                                                     _pool_slots(pool, stride, pool_slots),
-                                                    _dev_ptr(slots, torch.int32), slots.numel(),
-                                                    _dev_ptr(states_out, torch.float32),
+                                                    _dev_ptr(slots, _Torch.i32), slots.numel(),
+                                                    _dev_ptr(states_out, f),
                                                     _stream(stream)), "stepq_temporal_dequantize_pool")
 
 
 def stepq_decode_step(plan: Plan, layer: int, pool, slots, q, k, v, beta, gate, y,
                       pool_slots=None, stream=None):
-    import torch
-    f = torch.float32
+    f = _f32()
     B = slots.numel()
     check(_lib.lib().stepq_decode_step(plan.handle, layer, _dev_ptr(pool),
                                        _pool_slots(pool, plan.slot_stride, pool_slots),
-                                       _dev_ptr(slots, torch.int32), B, _dev_ptr(q, f),
+                                       _dev_ptr(slots, _Torch.i32), B, _dev_ptr(q, f),
                                        _dev_ptr(k, f), _dev_ptr(v, f), _dev_ptr(beta, f),
                                        _dev_ptr(gate, f), _dev_ptr(y, f), _stream(stream)),
           "stepq_decode_step")
@@ -244,11 +273,10 @@ def stepq_decode_step(plan: Plan, layer: int, pool, slots, q, k, v, beta, gate, 
 
 def stepq_decode_readout(plan: Plan, layer: int, pool, slots, q, k, v, beta, gate, y, delta,
                          pool_slots=None, stream=None):
-    import torch
-    f = torch.float32
+    f = _f32()
     check(_lib.lib().stepq_decode_readout(plan.handle, layer, _dev_ptr(pool),
                                           _pool_slots(pool, plan.slot_stride, pool_slots),
-                                          _dev_ptr(slots, torch.int32), slots.numel(),
+                                          _dev_ptr(slots, _Torch.i32), slots.numel(),
                                           _dev_ptr(q, f), _dev_ptr(k, f), _dev_ptr(v, f),
                                           _dev_ptr(beta, f), _dev_ptr(gate, f), _dev_ptr(y, f),
                                           _dev_ptr(delta, f), _stream(stream)),
@@ -257,11 +285,10 @@ def stepq_decode_readout(plan: Plan, layer: int, pool, slots, q, k, v, beta, gat
 
 def stepq_decode_writeback(plan: Plan, layer: int, pool, slots, k, beta, gate, delta,
                            pool_slots=None, stream=None):
-    import torch
-    f = torch.float32
+    f = _f32()
     check(_lib.lib().stepq_decode_writeback(plan.handle, layer, _dev_ptr(pool),
                                             _pool_slots(pool, plan.slot_stride, pool_slots),
-                                            _dev_ptr(slots, torch.int32), slots.numel(),
+                                            _dev_ptr(slots, _Torch.i32), slots.numel(),
                                             _dev_ptr(k, f), _dev_ptr(beta, f), _dev_ptr(gate, f),
                                             _dev_ptr(delta, f), _stream(stream)),
           "stepq_decode_writeback")
@@ -269,12 +296,11 @@ def stepq_decode_writeback(plan: Plan, layer: int, pool, slots, k, beta, gate, d
 
 def stepq_fp32_decode_step(cfg: Config, layer: int, pool, slots, q, k, v, beta, gate, y,
                            pool_slots=None, stream=None):
-    import torch
-    f = torch.float32
+    f = _f32()
     c = cfg.c()
     ps = pool_slots if pool_slots is not None else pool.shape[0]
     check(_lib.lib().stepq_fp32_decode_step(C.byref(c), layer, _dev_ptr(pool, f), int(ps),
-                                            _dev_ptr(slots, torch.int32), slots.numel(),
+                                            _dev_ptr(slots, _Torch.i32), slots.numel(),
                                             _dev_ptr(q, f), _dev_ptr(k, f), _dev_ptr(v, f),
                                             _dev_ptr(beta, f), _dev_ptr(gate, f), _dev_ptr(y, f),
                                             _stream(stream)), "stepq_fp32_decode_step")
@@ -282,13 +308,12 @@ def stepq_fp32_decode_step(cfg: Config, layer: int, pool, slots, q, k, v, beta, 
 
 def stepq_fp32_exact_read_step(cfg: Config, layer: int, pool, read_pool, slots, q, k, v, beta, gate,
                                y, pool_slots=None, stream=None):
-    import torch
-    f = torch.float32
+    f = _f32()
     c = cfg.c()
     ps = pool_slots if pool_slots is not None else pool.shape[0]
     check(_lib.lib().stepq_fp32_exact_read_step(C.byref(c), layer, _dev_ptr(pool, f),
                                                 _dev_ptr(read_pool, f), int(ps),
-                                                _dev_ptr(slots, torch.int32), slots.numel(),
+                                                _dev_ptr(slots, _Torch.i32), slots.numel(),
                                                 _dev_ptr(q, f), _dev_ptr(k, f), _dev_ptr(v, f),
                                                 _dev_ptr(beta, f), _dev_ptr(gate, f), _dev_ptr(y, f),
                                                 _stream(stream)), "stepq_fp32_exact_read_step")
@@ -298,8 +323,7 @@ def stepq_prefill_fp32(cfg: Config, states, q, k, v, beta, gate, y, stream=None)
     """Chunked prefill over T tokens on FP32 states [B][Hv][128][128] (in place);
     q, k [B][T][Hk][128], v [B][T][Hv][128], beta [B][T][Hv], gate [B][T][Hv]
     or [B][T][Hv][128], y [B][T][Hv][128] out."""
-    import torch
-    f = torch.float32
+    f = _f32()
     c = cfg.c()
     B, T = int(q.shape[0]), int(q.shape[1])
     check(_lib.lib().stepq_prefill_fp32(C.byref(c), B, T, _dev_ptr(states, f), _dev_ptr(q, f),
@@ -315,35 +339,34 @@ def stepq_intb_slot_bytes(cfg: Config, bits: int) -> int:
 
 def stepq_intb_quantize_pool(cfg: Config, bits: int, layer: int, states, slots, pool,
                              pool_slots=None, stream=None):
-    import torch
+    f = _f32()
     c = cfg.c()
     ps = _pool_slots(pool, stepq_intb_slot_bytes(cfg, bits), pool_slots)
     check(_lib.lib().stepq_intb_quantize_pool(C.byref(c), bits, layer,
-                                              _dev_ptr(states, torch.float32),
-                                              _dev_ptr(slots, torch.int32), slots.numel(),
+                                              _dev_ptr(states, f),
+                                              _dev_ptr(slots, _Torch.i32), slots.numel(),
                                               _dev_ptr(pool), ps, _stream(stream)),
           "stepq_intb_quantize_pool")
 
 
 def stepq_intb_dequantize_pool(cfg: Config, bits: int, layer: int, pool, slots, states_out,
                                pool_slots=None, stream=None):
-    import torch
+    f = _f32()
     c = cfg.c()
     ps = _pool_slots(pool, stepq_intb_slot_bytes(cfg, bits), pool_slots)
     check(_lib.lib().stepq_intb_dequantize_pool(C.byref(c), bits, layer, _dev_ptr(pool), ps,
-                                                _dev_ptr(slots, torch.int32), slots.numel(),
-                                                _dev_ptr(states_out, torch.float32),
+                                                _dev_ptr(slots, _Torch.i32), slots.numel(),
+                                                _dev_ptr(states_out, f),
                                                 _stream(stream)), "stepq_intb_dequantize_pool")
 
 
 def stepq_intb_decode_step(cfg: Config, bits: int, layer: int, pool, slots, q, k, v, beta, gate,
                            y, pool_slots=None, stream=None):
-    import torch
-    f = torch.float32
+    f = _f32()
     c = cfg.c()
     ps = _pool_slots(pool, stepq_intb_slot_bytes(cfg, bits), pool_slots)
     check(_lib.lib().stepq_intb_decode_step(C.byref(c), bits, layer, _dev_ptr(pool), ps,
-                                            _dev_ptr(slots, torch.int32), slots.numel(),
+                                            _dev_ptr(slots, _Torch.i32), slots.numel(),
                                             _dev_ptr(q, f), _dev_ptr(k, f), _dev_ptr(v, f),
                                             _dev_ptr(beta, f), _dev_ptr(gate, f), _dev_ptr(y, f),
                                             _stream(stream)), "stepq_intb_decode_step")
@@ -351,41 +374,40 @@ def stepq_intb_decode_step(cfg: Config, bits: int, layer: int, pool, slots, q, k
 
 def stepq_calib_observe(cfg: Config, layer: int, q, k, beta, gate, omega_sum, logret_sum,
                         stream=None):
-    import torch
-    f = torch.float32
+    f = _f32()
     c = cfg.c()
     check(_lib.lib().stepq_calib_observe(C.byref(c), layer, _dev_ptr(q, f), _dev_ptr(k, f),
                                          _dev_ptr(beta, f), _dev_ptr(gate, f), q.shape[0],
-                                         _dev_ptr(omega_sum, torch.float64),
-                                         _dev_ptr(logret_sum, torch.float64), _stream(stream)),
+                                         _dev_ptr(omega_sum, _Torch.f64),
+                                         _dev_ptr(logret_sum, _Torch.f64), _stream(stream)),
           "stepq_calib_observe")
 
 
 def stepq_calib_distortion(cfg: Config, layer: int, w, pivot_rows, states, acc, stream=None):
-    import torch
+    f = _f32()
     c = cfg.c()
-    check(_lib.lib().stepq_calib_distortion(C.byref(c), layer, _dev_ptr(w, torch.float32),
-                                            _dev_ptr(pivot_rows, torch.uint8),
-                                            _dev_ptr(states, torch.float32), states.shape[0],
-                                            _dev_ptr(acc, torch.float64), _stream(stream)),
+    check(_lib.lib().stepq_calib_distortion(C.byref(c), layer, _dev_ptr(w, f),
+                                            _dev_ptr(pivot_rows, _Torch.u8),
+                                            _dev_ptr(states, f), states.shape[0],
+                                            _dev_ptr(acc, _Torch.f64), _stream(stream)),
           "stepq_calib_distortion")
 
 
 def stepq_validate_slots(slots, pool_slots: int, scratch, status_out, stream=None):
-    import torch
-    check(_lib.lib().stepq_validate_slots(_dev_ptr(slots, torch.int32), slots.numel(),
-                                          int(pool_slots), _dev_ptr(scratch, torch.int32),
-                                          _dev_ptr(status_out, torch.int32), _stream(stream)),
+    _f32()
+    check(_lib.lib().stepq_validate_slots(_dev_ptr(slots, _Torch.i32), slots.numel(),
+                                          int(pool_slots), _dev_ptr(scratch, _Torch.i32),
+                                          _dev_ptr(status_out, _Torch.i32), _stream(stream)),
           "stepq_validate_slots")
 
 
 def stepq_validate_slots_noalloc(slots, pool_slots: int, status_out, stream=None):
     """stepq_validate_slots without a scratch argument: the library keeps the
     bitmap in a fixed device array (pool_slots <= 1,048,576) and allocates nothing."""
-    import torch
-    check(_lib.lib().stepq_validate_slots_noalloc(_dev_ptr(slots, torch.int32), slots.numel(),
+    _f32()
+    check(_lib.lib().stepq_validate_slots_noalloc(_dev_ptr(slots, _Torch.i32), slots.numel(),
                                                   int(pool_slots),
-                                                  _dev_ptr(status_out, torch.int32),
+                                                  _dev_ptr(status_out, _Torch.i32),
                                                   _stream(stream)),
           "stepq_validate_slots_noalloc")
 
@@ -423,7 +445,7 @@ def stepq_calibrate_from_trace(cfg: Config, q, k, v, beta, gate, every: int, str
     v [L][T][n][Hv][128], beta [L][T][n][Hv], gate [L][T][n][Hv] or [L][T][n][Hv][128]),
     all in the library (stepq_calibrate_from_trace); the workspace comes from torch."""
     import torch
-    f = torch.float32
+    f = _f32()
     L, T, n = q.shape[0], q.shape[1], q.shape[2]
     c = cfg.c()
     lib = _lib.lib()
