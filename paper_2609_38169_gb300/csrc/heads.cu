@@ -178,32 +178,39 @@ __device__ __forceinline__ void store_block(uint8_t *p, const uint32_t (&wd)[2 *
         *(uint4 *)(p + 512 * k) = make_uint4(wd[4 * k], wd[4 * k + 1], wd[4 * k + 2], wd[4 * k + 3]);
 }
 
-// Scale of the high code of a pair as placed by code_pair (2^B, or 1 for B = 8).
+// Placement of a code pair in float mantissas: code u in bits s.. s+B-1 under the
+// exponent of 2^(23-s) reads 2^(23-s) + u. The low code sits at s = kSlot, the high
+// one at kSlot + B (B = 8: both at kSlot). With s >= 12 - B the constant
+// c (2^(23-s) + 2^(B-1)) of an FP16 c has at most 24 significant bits, so that one
+// fma reconstructs c q exactly.
 template <int B>
-__host__ __device__ constexpr float hi_scale() { return B == 8 ? 1.0f : 1.0f / (float)(1 << B); }
+struct Code {
+    static constexpr int kSlot = B == 2 ? 12 : 8;
+    static constexpr int kHi = B == 8 ? kSlot : kSlot + B;
+    static_assert(kSlot >= 12 - B && kHi + B <= 23, "codes inside the mantissa, exact offsets");
+    __host__ __device__ static constexpr float base(int s) { return (float)(1 << (23 - s)) + (float)(1 << (B - 1)); }
+    __host__ __device__ static constexpr uint32_t bits(int s) { return (uint32_t)(127 + 23 - s) << 23; }
+};
 
-// Codes 2m and 2m+1 of chunk c of a block as the bit patterns of the floats
-// 1.5*2^23 + u_lo and 1.5*2^23 + u_hi * 2^B (B = 8: both at the bottom): the
-// codes are dropped into the zero low mantissa bits of the constant, one logic
-// op each (after at most one shift per pair).
+// Codes 2m and 2m+1 of chunk c of a block as floats (Code): one logic op each after at
+// most one shift per pair.
 template <int B>
 __device__ __forceinline__ uint64_t code_pair(const uint32_t (&wd)[2 * B], int c, int m) {
     constexpr int W = B / 2;                  // words per chunk
+    using K = Code<B>;
     if (B == 8) {
         const uint32_t w = wd[c * W + (m >> 1)];
-        const uint32_t sel = 0x7650u + 2u * (uint32_t)(m & 1);
-        return u2pair(__byte_perm(w, kMagicBits, sel), __byte_perm(w, kMagicBits, sel + 1u));
+        const uint32_t sel = 0x7604u + 0x20u * (uint32_t)(m & 1);       // the code into byte 1
+        return u2pair(__byte_perm(w, K::bits(8), sel), __byte_perm(w, K::bits(8), sel + 0x10u));
     }
     constexpr uint32_t mask = (1u << B) - 1u;
     const int p = 2 * m * B, k = c * W + (p >> 5), s = p & 31;
     uint32_t win;
-    if (s == 0)
-        win = wd[k];
-    else if (s + 2 * B <= 32)
-        win = wd[k] >> s;
+    if (s + 2 * B > 32)
+        win = __funnelshift_r(wd[k], wd[k + 1], s - K::kSlot);
     else
-        win = __funnelshift_r(wd[k], wd[k + 1], s);
-    return u2pair(and_or(win, mask, kMagicBits), and_or(win, mask << B, kMagicBits));
+        win = s >= K::kSlot ? wd[k] >> (s - K::kSlot) : wd[k] << (K::kSlot - s);
+    return u2pair(and_or(win, mask << K::kSlot, K::bits(K::kSlot)), and_or(win, mask << K::kHi, K::bits(K::kHi)));
 }
 
 // 16 offset-binary codes given as the float bit patterns 0x4B400000 | u_r,
@@ -443,15 +450,12 @@ __device__ __forceinline__ void load_tile(const T &t, const uint8_t *page, uint6
                             (uint16_t)(c4.y >> 16)};
 #pragma unroll
     for (int c = 0; c < 4; c++) {
-        // f = 1.5*2^23 + u s (s = 1 or the pair's high scale): fma(f, c/s, -1.5*2^23 c/s)
-        // = c u exactly (c fp16 and normal, u < 2^8: 19 significant bits; the
-        // offset has 12), and c u - c 2^(B-1) = c q is exact as well.
+        // f = 2^(23-s) + u: fma(f, c, -c (2^(23-s) + 2^(B-1))) = c q exactly (Code)
+        using K = Code<B>;
         const uint64_t cj = f2s(f16_val(ch[c]));
-        const uint64_t cc = fmul2(cj, f2(1.0f, hi_scale<B>()));
-        const uint64_t oc = fmul2(cc, f2s(-kMagic));
-        const uint64_t bc = fmul2(cj, f2s(-(float)(1 << (B - 1))));
+        const uint64_t oc = fmul2(cj, f2(-K::base(K::kSlot), -K::base(K::kHi)));
 #pragma unroll
-        for (int m = 0; m < 8; m++) x2[m][c] = fadd2(ffma2(code_pair<B>(wd, c, m), cc, oc), bc);
+        for (int m = 0; m < 8; m++) x2[m][c] = ffma2(code_pair<B>(wd, c, m), cj, oc);
     }
     }
 }
