@@ -68,6 +68,12 @@ __device__ __forceinline__ void cp_async_mbar_arrive(uint64_t *bar) {
     asm volatile("cp.async.mbarrier.arrive.shared::cta.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
+// The same, zero-filled instead of read when !valid.
+__device__ __forceinline__ void cp_async16_or_zero(void *dst_smem, const void *src_gmem, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst_smem)), "l"(src_gmem),
+                 "r"(valid ? 16 : 0)
+                 : "memory");
+}
 // This thread's cp.async copies have landed (a CTA barrier then shows them to all).
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 

@@ -14,26 +14,44 @@
 // and the state after the chunk is S_C = G_C S_0 + K_bar^T W, K_bar = K g_C / g.
 //
 // Every product runs on the tensor cores (tcgen05, kind::tf32) in split
-// precision: an fp32 operand is a TF32 head plus its remainder, and a product
-// is head*head + head*rest + rest*head (the rest*rest term is below fp32
-// rounding of the accumulation), which keeps fp32 accuracy. The state stays
-// in tensor memory as S^T (lane j = value column, column i = key row):
-//   P0  [K~ ; Q~] K^T        -> A, Bm      M = 128 (64 used), N = 32, K = 128, A, B in smem
-//   P1  S_0^T [K~ ; Q~]^T    -> [K~ S_0 ; Q~ S_0]^T    M = 128, N = 64, K = 128, A in tmem
-//   P2  S^T += W^T K_bar                               M = 128, N = 128, K = 32, A in tmem
-//   P3  (Q~ S_0)^T += W^T Bm^T  -> Y^T                 M = 128, N = 32, K = 32, A in tmem
-// Shared-memory operands are K-major core matrices (8 rows x 16 bytes). The
-// FMA pipe keeps the element-wise work, the triangular solve (I + A) W = R
-// (one value column per thread) and the scaling of S by g_C.
+// precision: an fp32 operand is its TF32 head, which is all the tensor core reads of
+// it, plus a remainder, and a product is head*head + head*rest + rest*head (P0 and P1
+// also take rest*rest), which keeps fp32 accuracy. The state stays in tensor memory as
+// S^T (lane j = value column, column i = key row):
+//   P0  [Q~ ; K~] K^T        -> Bm, A      M = 128, N = 64, K = 128, A, B in smem
+//   P1  S_0^T [Q~ ; K~]^T    -> [Q~ S_0 ; K~ S_0]^T    M = 128, N = 128, K = 128, A in tmem
+//   P2  S^T += W^T K_bar and Y^T = (Q~ S_0)^T + W^T Bm^T   M = 128, N = 160, K = 32, A in tmem
+// An MMA with M = 128 takes N / 2 cycles, but not less than the 45 that its issue takes,
+// so operands are stacked until N is at least 128 where they can be: P0's A rows and P1's B rows
+// are [Q~ ; K~] (64) over its rests (64), P0's B rows K^ (32) over its rests (32), P2's
+// K_bar^T (128) over Bm (32). The partial products of stacked rests land in columns
+// (or, P0, lanes) of their own and are added when they are read. Shared-memory
+// operands are K-major core matrices (8 rows x 16 bytes). The FMA pipe keeps the
+// element-wise work, the triangular solve (I + A) W = R (one value column per thread)
+// and the scaling of S by g_C.
 //
-// One CTA (256 threads, 8 warps) per SM, persistent over (slot, value head)
-// items; it owns all 512 tensor-memory columns:
-//   [0, 128) S^T fp32 | [128, 256) S^T head | [256, 384) S^T rest |
-//   [384, 416) (K~ S_0)^T | [416, 448) (Q~ S_0)^T, then Y^T |
-//   [448, 480) P0 result, then W^T head | [480, 512) W^T rest.
-// Warps w and w + 4 share tensor-memory lanes 32 (w % 4) ..: the first four
-// warps solve for W while the last four scale the state by g_C. While P2 and
-// P3 run, all warps prepare the next chunk's operands.
+// One persistent CTA of 20 warps per SM; it owns all 512 tensor-memory columns:
+//   [0, 128) S^T | [128, 160) Y^T | [160, 192) (K~ S_0)^T | [192, 256) the rests' part of
+//   both | [256, 384) S^T rest | [384, 448) P0 result | [448, 480) W^T | [480, 512) W^T rest
+// The chunks of a head are a serial chain P1 -> solve -> P2 -> state rest, so the time
+// of a chunk is that chain's latency, and everything else runs beside it:
+//   warps 0-7   the chain: A and Bm from P0 (under P1), solve for W, scale S, its rest;
+//               a chunk's y leaves under the next chunk's P1
+//   warps 8-15  the next chunk's operands: loads, cumulative gates, products and rests,
+//               written as soon as the products of this chunk have read theirs
+//   warp 16     issues the MMAs (an issuing thread waits on the tensor pipe's queue),
+//               P0 of the next chunk right after P2, under the outputs' and state's reads
+// With 8 warps doing all of it in turn a chunk took 17,700 cycles: 6,700 the operands,
+// 5,500 waiting on P0 and P1 (96 MMAs then, 48 now), 2,200 the solve, 1,500 the
+// outputs. It takes 8,700 now: 3,100 P0's end and P1, 2,600 the solve (which shares the
+// SM's issue slots with warps 8-15), 1,300 P2, 1,600 the outputs' and the state's reads.
+// 128 slots x 32 heads x 512 tokens: 4.05 ms then, 1.98 ms now.
+//
+// Hand-over, all by mbarriers, one phase a chunk, every wait bounded: `full1` (warps
+// 8-15: Q~, K~, K^, V, beta, g_C) starts P0, which completes `p0`; `ready` (warps 0-7: S
+// and its rest, Y read) starts P1, which completes `p1`; `wready` (warps 0-7: W, Bm,
+// scaled S) and `full2` (warps 8-15: K_bar) start P2, which completes `p2`. Warps 8-15
+// refill Q~, K~, K^ after p1 and K_bar after p2; V, beta and g_C have two buffers.
 #include "async.cuh"
 #include "device.cuh"
 #include "internal.h"
@@ -44,63 +62,76 @@ namespace stepq {
 namespace pf {
 
 constexpr int C = 32;                                  // tokens per chunk
-constexpr uint32_t kColS = 0, kColSh = 128, kColSl = 256, kColX = 384, kColY = 416, kColP0 = 448,
-                   kColWh = 448, kColWl = 480;
+constexpr int kGroup = 256;                            // threads of warps 0-7 and of warps 8-15
+constexpr int kBlock = 2 * kGroup + 128;
+// Registers a thread: 96 at launch (20 warps), then the shares of the three groups.
+constexpr int kRegs = 96, kRegsChain = 120, kRegsIssue = 48;
+static_assert(kGroup * (kRegsChain + kRegs) + 128 * kRegsIssue <= kBlock * kRegs, "register shares");
+constexpr uint32_t kColS = 0, kColY = 128, kColX = 160, kColYl = 192, kColXl = 224, kColSl = 256, kColP0 = 384,
+                   kColW = 448, kColWl = 480;
 constexpr uint32_t kCols = 512;
-constexpr uint32_t kIdescP0 = tc::idesc_tf32(128, 32);
-constexpr uint32_t kIdescP1 = tc::idesc_tf32(128, 64);
-constexpr uint32_t kIdescP2 = tc::idesc_tf32(128, 128);
-constexpr uint32_t kIdescP3 = tc::idesc_tf32(128, 32);
+constexpr uint32_t kIdescP0 = tc::idesc_tf32(128, 64);
+constexpr uint32_t kIdescP1 = tc::idesc_tf32(128, 128), kIdescP1l = tc::idesc_tf32(128, 64);
+constexpr uint32_t kIdescP2 = tc::idesc_tf32(128, 160);
 
-// Shared-memory operands: K-major core matrices of 8 rows x 4 fp32 (128 B),
-// the core matrices of one row group 144 B apart along K (16 B of padding each,
-// so that a warp storing 32 consecutive K elements of one row hits 32 banks),
-// row groups kSbo128 / kSbo32 apart for K = 128 / 32.
-constexpr int kLbo = 144;
-constexpr int kSbo128 = 32 * kLbo;                     // 4608
-constexpr int kSbo32 = 8 * kLbo + 16;                  // 1168: 16-byte rows of 8 row groups in distinct banks
-// P0 reads 128 rows of A from B1: rows 64..127 fall on B1l and B3 (valid
-// memory; their results are unused).
-constexpr int kOffB1h = 0;                             // [K~ ; Q~] head: 64 rows x K 128
-constexpr int kOffB1l = kOffB1h + 8 * kSbo128;         // rest
-constexpr int kOffB3h = kOffB1l + 8 * kSbo128;         // K^ head: 32 rows (s) x K 128
-constexpr int kOffB3l = kOffB3h + 4 * kSbo128;
-constexpr int kOffB2h = kOffB3l + 4 * kSbo128;         // K_bar^T head: 128 rows (i) x K 32 (t)
-constexpr int kOffB2l = kOffB2h + 16 * kSbo32;
-constexpr int kOffB4h = kOffB2l + 16 * kSbo32;         // Bm head: 32 rows (t) x K 32 (s)
-constexpr int kOffB4l = kOffB4h + 4 * kSbo32;
-constexpr int kOffV = kOffB4l + 4 * kSbo32;            // float [C][128] V
-constexpr int kOffG = kOffV + C * 128 * 4;             // float [C][128] cumulative gates
-constexpr int kOffA = kOffG + C * 128 * 4;             // float [C][C] A^T: row s holds A_ts over t (t > s)
-constexpr int kOffBeta = kOffA + C * C * 4;            // float [C]
-constexpr int kOffBar = kOffBeta + C * 4;              // uint64 mbarrier
-constexpr int kOffTmem = kOffBar + 8;                  // u32 tensor-memory base
-constexpr int kSmem = kOffTmem + 8;
-static_assert(kOffB1l + 16 * kSbo128 <= kSmem, "P0's unused A rows must stay inside shared memory");
+// Shared-memory operands: K-major core matrices of 8 rows x 4 fp32 (128 B). Strides are
+// chosen for the stores alone (the tensor core's time does not depend on them): with
+// K = 128 the matrices are back to back and a quarter warp stores 8 tokens of one; with
+// K = 32 they are 144 B apart along K and 1184 B between row groups, so that a warp's
+// scalar stores (8 tokens x 4 channels) hit 32 banks.
+constexpr int kLbo128 = 128, kSbo128 = 32 * kLbo128;
+constexpr int kLbo32 = 144, kSbo32 = 8 * kLbo32 + 32;
+constexpr int kVRow = 132;                             // padded row of V
+constexpr int kOffB1 = 0;                              // [Q~ ; K~] 64 rows x K 128, then its rests
+constexpr int kOffB1l = kOffB1 + 8 * kSbo128;
+constexpr int kOffB3 = kOffB1l + 8 * kSbo128;          // K^ 32 rows (s) x K 128, then its rests
+constexpr int kOffB3l = kOffB3 + 4 * kSbo128;
+constexpr int kOffB2 = kOffB3l + 4 * kSbo128;          // K_bar^T 128 rows (i) x K 32 (t), then Bm 32 rows (t) x K 32 (s)
+constexpr int kOffB4 = kOffB2 + 16 * kSbo32;
+constexpr int kOffB2l = kOffB4 + 4 * kSbo32;           // the rests of both
+constexpr int kOffB4l = kOffB2l + 16 * kSbo32;
+constexpr int kOffV = kOffB4l + 4 * kSbo32;            // float [2][C][kVRow] V
+constexpr int kOffGc = kOffV + 2 * C * kVRow * 4;      // float [2][128] g_C
+constexpr int kOffBeta = kOffGc + 2 * 128 * 4;         // float [2][C]
+constexpr int kOffA = kOffBeta + 2 * C * 4;            // float [C][C] -A^T: row s holds -A_ts over t (t > s)
+constexpr int kFRow = C + 4;                           // padded row of F
+constexpr int kOffF = kOffA + C * C * 4;               // float [64][kFRow] P0 partials of the rest rows
+constexpr int kOffQK = kOffF + 64 * kFRow * 4;         // float4 [8][kGroup] the next chunk's q and k, by thread
+constexpr int kOffBar = kOffQK + 8 * kGroup * 16;        // uint64 [8] mbarriers
+constexpr int kOffTmem = kOffBar + 64;                 // u32 tensor-memory base
+constexpr int kSmem = kOffTmem + 16;
+static_assert(kSmem <= kSmemMax, "one CTA's shared memory");
+enum { kReady, kFull1, kP0, kP1, kWready, kFull2, kP2, kDrain };
 
-// Byte offset of element (row r, k) of a K-major operand with row groups `sbo` apart.
-__device__ __forceinline__ int core_off(int r, int k, int sbo) {
-    return (r >> 3) * sbo + (k >> 2) * kLbo + (r & 7) * 16 + (k & 3) * 4;
+// Byte offset of element (row r, k) of a K-major operand.
+__device__ __forceinline__ int off128(int r, int k) { return (r >> 3) * kSbo128 + (k >> 2) * kLbo128 + (r & 7) * 16; }
+__device__ __forceinline__ int off32(int r, int k) {
+    return (r >> 3) * kSbo32 + (k >> 2) * kLbo32 + (r & 7) * 16 + (k & 3) * 4;
 }
 
-__device__ __forceinline__ void put_split(uint8_t *hi_base, uint8_t *lo_base, int off, float x) {
-    float hi, lo;
-    tc::split_tf32(x, hi, lo);
-    *(float *)(hi_base + off) = hi;
-    *(float *)(lo_base + off) = lo;
-}
-// Four consecutive K elements of one row (off 16-byte aligned).
-__device__ __forceinline__ void put_split4(uint8_t *hi_base, uint8_t *lo_base, int off, float4 x) {
-    float4 hi, lo;
-    tc::split_tf32(x.x, hi.x, lo.x);
-    tc::split_tf32(x.y, hi.y, lo.y);
-    tc::split_tf32(x.z, hi.z, lo.z);
-    tc::split_tf32(x.w, hi.w, lo.w);
-    *(float4 *)(hi_base + off) = hi;
-    *(float4 *)(lo_base + off) = lo;
+// Four consecutive K elements of one row (off 16-byte aligned) and their rests.
+__device__ __forceinline__ void put4(uint8_t *base, uint8_t *rest, int off, float4 x) {
+    *(float4 *)(base + off) = x;
+    *(float4 *)(rest + off) =
+        make_float4(tc::tf32_rest(x.x), tc::tf32_rest(x.y), tc::tf32_rest(x.z), tc::tf32_rest(x.w));
 }
 __device__ __forceinline__ float4 mul4(float4 a, float4 b) {
     return make_float4(a.x * b.x, a.y * b.y, a.z * b.z, a.w * b.w);
+}
+__device__ __forceinline__ float rcp(float x) {          // within 1 ulp
+    float d;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(d) : "f"(x));
+    return d;
+}
+// Barrier over the 256 threads of warps 0-7; returns the OR of their predicates.
+__device__ __forceinline__ bool group_any(bool p) {
+    uint32_t r;
+    asm volatile(
+        "{ .reg .pred p, q; setp.ne.u32 p, %1, 0; barrier.cta.red.or.pred q, 1, 256, p; selp.u32 %0, 1, 0, q; }"
+        : "=r"(r)
+        : "r"((uint32_t)p)
+        : "memory");
+    return r != 0;
 }
 
 struct Args {
@@ -110,23 +141,407 @@ struct Args {
     unsigned int *err;
 };
 
-__global__ void __launch_bounds__(kThreads, 1) prefill_kernel(Args a) {
+// Cumulative gates of a chunk: this thread's float4 of four channels at tokens 8 m + tl
+// (m = 0..3, tl = lane & 7), multiplied up over the tokens by a scan over the 8 lanes
+// of a token block and the blocks before it; kept above 1e-30 so that K / g stays
+// finite. Returns g_C.
+__device__ __forceinline__ float4 scan_channels(float4 (&g)[4], int tl) {
+    const auto up = [&](float x, int o) {
+        const float y = __shfl_up_sync(0xffffffffu, x, o, 8);
+        return tl >= o ? x * y : x;
+    };
+    const auto floor4 = [](float4 a, float4 b) {
+        return make_float4(fmaxf(a.x * b.x, 1e-30f), fmaxf(a.y * b.y, 1e-30f), fmaxf(a.z * b.z, 1e-30f),
+                           fmaxf(a.w * b.w, 1e-30f));
+    };
+    float4 run = make_float4(1.f, 1.f, 1.f, 1.f);
+#pragma unroll
+    for (int m = 0; m < 4; m++) {
+#pragma unroll
+        for (int o = 1; o < 8; o *= 2) g[m] = make_float4(up(g[m].x, o), up(g[m].y, o), up(g[m].z, o), up(g[m].w, o));
+        const float4 all = make_float4(__shfl_sync(0xffffffffu, g[m].x, 7, 8), __shfl_sync(0xffffffffu, g[m].y, 7, 8),
+                                       __shfl_sync(0xffffffffu, g[m].z, 7, 8), __shfl_sync(0xffffffffu, g[m].w, 7, 8));
+        g[m] = floor4(run, g[m]);
+        run = floor4(run, all);
+    }
+    return run;
+}
+
+// Warps 8-15: the operands of this CTA's chunks, in order. Warp pw holds channels
+// 16 pw .. +15; lane l holds channels 16 pw + 4 (l >> 3) .. +3 at tokens 8 m + (l & 7),
+// so that a load covers 64-byte pieces of 8 tokens, a quarter warp's operand store one
+// core matrix, and the gates' product over the tokens stays inside the warp. The inputs
+// come by cp.async, a thread's own q and k into a place of its own and V where the solve
+// reads it (loads into registers, 64 of them, spilled as they arrived and held the warps
+// for their latency). Missing tokens of a ragged tail are the identity step (gate 1, beta
+// 0, zero k, q, v).
+__device__ __forceinline__ bool produce(const Args &a, uint8_t *smem, uint64_t *bars) {
+    uint8_t *B1 = smem + kOffB1, *B1l = smem + kOffB1l, *B2 = smem + kOffB2, *B2l = smem + kOffB2l;
+    uint8_t *B3 = smem + kOffB3, *B3l = smem + kOffB3l;
+    const int l = threadIdx.x & 31, tl = l & 7, pw = (threadIdx.x - kGroup) >> 5, c4 = 16 * pw + 4 * (l >> 3);
+    const int grp = a.Hv / a.Hk;
+    float4 *qk = (float4 *)(smem + kOffQK) + (threadIdx.x - kGroup);
+    float4 g[4];
+    float ds = 1.f, bt = 0.f;
+    int fn = 0;
+    // q, k, gates and beta of a chunk; its V (buffer vb) once that buffer is free
+    const auto fetch = [&](int item, int c0) {
+        const int b = item / a.Hv, h = item - b * a.Hv, hk = h / grp;
+        fn = min(C, a.T - c0);
+        const size_t tok0 = (size_t)b * a.T + c0, tok = tok0 + min(l, fn - 1);
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            const bool in = 8 * m + tl < fn;
+            const size_t t = tok0 + (in ? 8 * m + tl : 0), ke = (t * a.Hk + hk) * 128 + c4;
+            cp_async16_or_zero(&qk[2 * m * kGroup], &a.q[ke], in);
+            cp_async16_or_zero(&qk[(2 * m + 1) * kGroup], &a.k[ke], in);
+            if (a.gate_per_row) g[m] = *(const float4 *)&a.gate[(t * a.Hv + h) * 128 + c4];
+        }
+        if (!a.gate_per_row) ds = a.gate[tok * a.Hv + h];
+        if (pw == 0) bt = a.beta[tok * a.Hv + h];
+    };
+    const auto fetch_v = [&](int item, int c0, uint32_t vb) {
+        const int b = item / a.Hv, h = item - b * a.Hv, n = min(C, a.T - c0);
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            const int t = 8 * m + tl;
+            const size_t tok = (size_t)b * a.T + c0 + (t < n ? t : 0);
+            cp_async16_or_zero(smem + kOffV + ((vb * C + t) * kVRow + c4) * 4, &a.v[(tok * a.Hv + h) * 128 + c4], t < n);
+        }
+    };
+    const auto wait = [&](int bar, uint32_t ph) {
+        return (bool)__all_sync(0xffffffffu, mbar_wait(&bars[bar], ph, pipe::kWaitCycles));
+    };
+    int item = blockIdx.x, c0 = 0;
+    if (item < a.items) {
+        fetch(item, 0);
+        fetch_v(item, 0, 0);
+    }
+    for (uint32_t n = 0; item < a.items; n++) {
+        const uint32_t buf = n & 1u, prev = buf ^ 1u;      // prev: parity of chunk n - 1's phases
+        float4 gC;
+        if (a.gate_per_row) {
+#pragma unroll
+            for (int m = 0; m < 4; m++)
+                if (8 * m + tl >= fn) g[m] = make_float4(1.f, 1.f, 1.f, 1.f);
+            gC = scan_channels(g, tl);
+        } else {                                           // lane l: token l
+            float d = l < fn ? ds : 1.f;
+#pragma unroll
+            for (int o = 1; o < 32; o *= 2) {
+                const float y = __shfl_up_sync(0xffffffffu, d, o);
+                d = l >= o ? d * y : d;
+            }
+            d = fmaxf(d, 1e-30f);
+            const float dC = __shfl_sync(0xffffffffu, d, 31);
+            gC = make_float4(dC, dC, dC, dC);
+#pragma unroll
+            for (int m = 0; m < 4; m++) {
+                const float x = __shfl_sync(0xffffffffu, d, 8 * m + tl);
+                g[m] = make_float4(x, x, x, x);
+            }
+        }
+        cp_async_wait_all();                               // q, k and V
+        // P0 of the chunk before has read K^, its P1 Q~ and K~; beta and g_C of two
+        // chunks ago are used up (S's rest was formed before that P1 started).
+        if (n > 0 && !wait(kP0, prev)) return false;
+        float4 kb[4];                                      // K_bar at the thread's tokens
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            float4 kr = make_float4(rcp(g[m].x), 0.f, 0.f, 0.f);
+            kr.y = a.gate_per_row ? rcp(g[m].y) : kr.x;
+            kr.z = a.gate_per_row ? rcp(g[m].z) : kr.x;
+            kr.w = a.gate_per_row ? rcp(g[m].w) : kr.x;
+            kr = mul4(qk[(2 * m + 1) * kGroup], kr);
+            put4(B3, B3l, off128(8 * m + tl, c4), kr);                              // K^
+            kb[m] = mul4(kr, gC);
+        }
+        if (n > 0 && !wait(kP1, prev)) return false;
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            const int t = 8 * m + tl;
+            put4(B1, B1l, off128(t, c4), mul4(g[m], qk[2 * m * kGroup]));           // Q~
+            put4(B1, B1l, off128(C + t, c4), mul4(g[m], qk[(2 * m + 1) * kGroup])); // K~
+        }
+        if (tl == 0) *(float4 *)(smem + kOffGc + (buf * 128 + c4) * 4) = gC;
+        if (pw == 0) ((float *)(smem + kOffBeta))[buf * C + l] = l < fn ? bt : 0.f;
+        fence_async_smem();
+        mbar_arrive(&bars[kFull1]);
+        c0 += C;
+        if (c0 >= a.T) {
+            item += gridDim.x;
+            c0 = 0;
+        }
+        if (item < a.items) fetch(item, c0);
+        // P2 of the chunk before has read K_bar.
+        if (n > 0 && !wait(kP2, prev)) return false;
+#pragma unroll
+        for (int m = 0; m < 4; m++) {
+            const float e4[4] = {kb[m].x, kb[m].y, kb[m].z, kb[m].w};
+#pragma unroll
+            for (int e = 0; e < 4; e++) {
+                const int o = off32(c4 + e, 8 * m + tl);
+                *(float *)(B2 + o) = e4[e];
+                *(float *)(B2l + o) = tc::tf32_rest(e4[e]);
+            }
+        }
+        fence_async_smem();
+        mbar_arrive(&bars[kFull2]);
+        if (item < a.items) fetch_v(item, c0, prev);       // V of the chunk before is used up
+    }
+    return true;
+}
+
+// Warp 16, one thread: the MMAs of this CTA's chunks.
+__device__ __forceinline__ bool issue_mma(const Args &a, uint8_t *smem, uint64_t *bars, uint32_t tm) {
+    // Descriptors of each operand's first K step; a step of 8 adds 2 core matrices. (A loop
+    // that built its descriptors took up to 110 cycles an MMA.)
+    const uint64_t d1 = tc::sdesc(smem + kOffB1, kLbo128, kSbo128), d3 = tc::sdesc(smem + kOffB3, kLbo128, kSbo128);
+    const uint64_t d2 = tc::sdesc(smem + kOffB2, kLbo32, kSbo32), d2l = tc::sdesc(smem + kOffB2l, kLbo32, kSbo32);
+    constexpr uint64_t k128 = 2 * kLbo128 / 16, k32 = 2 * kLbo32 / 16;
+    const int per = (a.T + C - 1) / C, mine = (a.items - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    const long long chunks = (long long)per * mine;
+    bool ok = true;
+    const auto p0 = [&](uint32_t ph) {
+        ok = mbar_wait(&bars[kFull1], ph, pipe::kWaitCycles);
+        if (!ok) return;
+        tc::fence_after();
+#pragma unroll 1
+        for (int s = 0; s < 16; s++)
+            tc::mma_tf32_ss(tm + kColP0, d1 + s * k128, d3 + s * k128, kIdescP0, s > 0 ? 1u : 0u);
+        tc::commit(&bars[kP0]);
+    };
+    p0(0);
+    for (long long n = 0; ok && n < chunks; n++) {
+        const uint32_t ph = (uint32_t)n & 1u;
+        if (!(ok = mbar_wait(&bars[kReady], ph, pipe::kWaitCycles))) break;
+        tc::fence_after();
+#pragma unroll 1
+        for (int s = 0; s < 16; s++) {
+            tc::mma_tf32_ts(tm + kColY, tm + kColS + 8 * s, d1 + s * k128, kIdescP1, s > 0 ? 1u : 0u);
+            tc::mma_tf32_ts(tm + kColY, tm + kColSl + 8 * s, d1 + s * k128, kIdescP1l, 1u);
+        }
+        tc::commit(&bars[kP1]);
+        ok = mbar_wait(&bars[kFull2], ph, pipe::kWaitCycles) && mbar_wait(&bars[kWready], ph, pipe::kWaitCycles);
+        if (!ok) break;
+        tc::fence_after();
+#pragma unroll 1
+        for (int s = 0; s < 4; s++) {
+            tc::mma_tf32_ts(tm + kColS, tm + kColW + 8 * s, d2 + s * k32, kIdescP2, 1u);
+            tc::mma_tf32_ts(tm + kColS, tm + kColW + 8 * s, d2l + s * k32, kIdescP2, 1u);
+            tc::mma_tf32_ts(tm + kColS, tm + kColWl + 8 * s, d2 + s * k32, kIdescP2, 1u);
+        }
+        tc::commit(&bars[kP2]);
+        if (n + 1 < chunks) p0(ph ^ 1u);
+    }
+    // every MMA has ended before the tensor memory is given back
+    tc::commit(&bars[kDrain]);
+    return mbar_wait(&bars[kDrain], 0, pipe::kWaitCycles) && ok;
+}
+
+// Warps 0-7: the chain of this CTA's chunks. Warps w and w + 4 share tensor-memory
+// lanes 32 (w % 4) ..; lane j = value column (and row of P0's result).
+__device__ __forceinline__ bool chain(const Args &a, uint8_t *smem, uint64_t *bars, uint32_t tm) {
+    uint8_t *B4 = smem + kOffB4, *B4l = smem + kOffB4l;
+    float *A = (float *)(smem + kOffA), *F = (float *)(smem + kOffF);
+    const int w = threadIdx.x >> 5, l = threadIdx.x & 31, quad = w & 3, half = w >> 2;
+    const int j = 32 * quad + l;
+    const uint32_t tl = tm + ((uint32_t)(32 * quad) << 16);   // this warp's lanes
+    uint32_t ph = 0;
+    bool ok = true;
+    float yv[16], *yp = nullptr;                          // the previous chunk's outputs
+    int yn = 0;
+    const auto store_y = [&]() {
+#pragma unroll
+        for (int e = 0; e < 16; e++)
+            if (e < yn) yp[(size_t)e * a.Hv * 128] = yv[e];
+    };
+    for (int item = blockIdx.x; item < a.items; item += gridDim.x) {
+        const int b = item / a.Hv, h = item - b * a.Hv;
+        float *Sg = a.states + (size_t)item * kN;
+        // S^T into tensor memory: this thread's lane j, the 64 key rows of its half.
+        {
+            float sv[64];
+#pragma unroll
+            for (int e = 0; e < 64; e++) sv[e] = Sg[(size_t)(64 * half + e) * 128 + j];
+            tc::st64(tl + kColS + 64 * half, sv);
+#pragma unroll
+            for (int e = 0; e < 64; e++) sv[e] = tc::tf32_rest(sv[e]);
+            tc::st64(tl + kColSl + 64 * half, sv);
+        }
+        for (int t0 = 0; t0 < a.T; t0 += C, ph ^= 1u) {
+            const int n = min(C, a.T - t0);               // tokens in this chunk (ragged tail)
+            const bool last = t0 + C >= a.T;
+            const float *V = (const float *)(smem + kOffV) + ph * C * kVRow;
+            const float *gC = (const float *)(smem + kOffGc) + ph * 128;
+            const float *bet = (const float *)(smem + kOffBeta) + ph * C;
+            tc::wait_st();
+            tc::fence_before();
+            // full1 first: its next phase then cannot end before this thread has seen this one
+            ok = mbar_wait(&bars[kFull1], ph, pipe::kWaitCycles) && ok;
+            mbar_arrive(&bars[kReady]);
+            store_y();
+            // P0's result, row r = lane: [Q~ ; K~] in lanes 0-63, its rests in 64-127;
+            // columns s over K^, 32 + s over its rests. This half takes columns
+            // 16 half .. +15.
+            ok = mbar_wait(&bars[kP0], ph, pipe::kWaitCycles) && ok;
+            tc::fence_after();
+            float d[16];
+            {
+                float e[16];
+                tc::ld16(tl + kColP0 + 16 * half, d);
+                tc::ld16(tl + kColP0 + 32 + 16 * half, e);
+#pragma unroll
+                for (int s = 0; s < 16; s++) d[s] += e[s];
+            }
+            if (quad >= 2) {
+#pragma unroll
+                for (int s = 0; s < 16; s += 4)
+                    *(float4 *)&F[(j - 64) * kFRow + 16 * half + s] = make_float4(d[s], d[s + 1], d[s + 2], d[s + 3]);
+            }
+            tc::fence_before();
+            if (group_any(!ok)) return false;
+            // Bm = lower (with diagonal) of Q~ K^T (row t = lane t), an operand, and
+            // A = strict lower of diag(beta) K~ K^T (row t = lane 32 + t), kept negated
+            // and transposed (a warp's store is part of one row of A^T).
+            if (quad < 2) {
+#pragma unroll
+                for (int s = 0; s < 16; s += 4) {
+                    const float4 f = *(const float4 *)&F[j * kFRow + 16 * half + s];
+                    d[s] += f.x;
+                    d[s + 1] += f.y;
+                    d[s + 2] += f.z;
+                    d[s + 3] += f.w;
+                }
+                if (quad == 1) {
+                    const float nb = -bet[l];
+#pragma unroll
+                    for (int e = 0; e < 16; e++) {
+                        const int s = 16 * half + e;
+                        A[s * C + l] = s < l ? nb * d[e] : 0.f;
+                    }
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 16; e += 4) {
+                        const int s = 16 * half + e;
+                        put4(B4, B4l, off32(l, s),
+                             make_float4(s <= l ? d[e] : 0.f, s + 1 <= l ? d[e + 1] : 0.f,
+                                         s + 2 <= l ? d[e + 2] : 0.f, s + 3 <= l ? d[e + 3] : 0.f));
+                    }
+                    fence_async_smem();
+                }
+            }
+            ok = mbar_wait(&bars[kP1], ph, pipe::kWaitCycles);
+            if (group_any(!ok)) return false;           // also: A visible, P0's columns free for W
+            tc::fence_after();
+            if (half == 0) {
+                // W = (I + A)^-1 diag(beta) (V - K~ S_0), value column j, by forward
+                // substitution in column order: once w_s is final it is taken out
+                // of every later row, two rows an fma (independent updates, so the
+                // dependent chain is one fma per token).
+                float x[32];
+                {
+                    float xl[32];
+                    tc::ld32(tl + kColX, x);
+                    tc::ld32(tl + kColXl, xl);
+#pragma unroll
+                    for (int t = 0; t < C; t++) x[t] += xl[t];
+                }
+                uint64_t wv[16];
+#pragma unroll
+                for (int p = 0; p < 16; p++)
+                    wv[p] = f2(bet[2 * p] * (V[2 * p * kVRow + j] - x[2 * p]),
+                               bet[2 * p + 1] * (V[(2 * p + 1) * kVRow + j] - x[2 * p + 1]));
+#pragma unroll
+                for (int s = 0; s < C - 1; s++) {
+                    const uint64_t ws = f2s(s & 1 ? f2hi(wv[s >> 1]) : f2lo(wv[s >> 1]));
+#pragma unroll
+                    for (int t4 = (s + 1) / 4; t4 < C / 4; t4++) {    // row s of -A^T, four at a time
+                        const uint4 a4 = ((const uint4 *)(A + s * C))[t4];
+                        if (4 * t4 + 1 > s) wv[2 * t4] = ffma2(u2pair(a4.x, a4.y), ws, wv[2 * t4]);
+                        wv[2 * t4 + 1] = ffma2(u2pair(a4.z, a4.w), ws, wv[2 * t4 + 1]);
+                    }
+                }
+#pragma unroll
+                for (int p = 0; p < 16; p++) {
+                    x[2 * p] = f2lo(wv[p]);
+                    x[2 * p + 1] = f2hi(wv[p]);
+                }
+                tc::st32(tl + kColW, x);
+#pragma unroll
+                for (int t = 0; t < C; t++) x[t] = tc::tf32_rest(x[t]);
+                tc::st32(tl + kColWl, x);
+            } else {
+                // S^T <- S^T diag(g_C): key row i scaled by its cumulative gate.
+#pragma unroll 1
+                for (int c = 0; c < 128; c += 64) {
+                    float sv[64];
+                    tc::ld64(tl + kColS + c, sv);
+#pragma unroll
+                    for (int e = 0; e < 64; e += 4) {
+                        const float4 g = *(const float4 *)&gC[c + e];
+                        sv[e] *= g.x;
+                        sv[e + 1] *= g.y;
+                        sv[e + 2] *= g.z;
+                        sv[e + 3] *= g.w;
+                    }
+                    tc::st64(tl + kColS + c, sv);
+                }
+            }
+            tc::wait_st();
+            tc::fence_before();
+            mbar_arrive(&bars[kWready]);
+            ok = mbar_wait(&bars[kP2], ph, pipe::kWaitCycles);
+            tc::fence_after();
+            // Outputs: tokens 16 half .. 16 half + 15 of column j, stored once the next
+            // chunk can start.
+            tc::ld16(tl + kColY + 16 * half, yv);
+            {
+                float yl[16];
+                tc::ld16(tl + kColYl + 16 * half, yl);
+#pragma unroll
+                for (int e = 0; e < 16; e++) yv[e] += yl[e];
+            }
+            // The rest of the new state for the next chunk's P1, or the boundary state
+            // back to global memory.
+            {
+                float sv[64];
+                tc::ld64(tl + kColS + 64 * half, sv);
+                if (last) {
+#pragma unroll
+                    for (int e = 0; e < 64; e++) Sg[(size_t)(64 * half + e) * 128 + j] = sv[e];
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 64; e++) sv[e] = tc::tf32_rest(sv[e]);
+                    tc::st64(tl + kColSl + 64 * half, sv);
+                }
+            }
+            yp = a.y + (((size_t)b * a.T + t0 + 16 * half) * a.Hv + h) * 128 + j;
+            yn = n - 16 * half;
+        }
+    }
+    store_y();
+    return ok;
+}
+
+__global__ void __launch_bounds__(kBlock, 1) prefill_kernel(Args a) {
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t *B1h = smem + kOffB1h, *B1l = smem + kOffB1l, *B2h = smem + kOffB2h, *B2l = smem + kOffB2l;
-    uint8_t *B3h = smem + kOffB3h, *B3l = smem + kOffB3l, *B4h = smem + kOffB4h, *B4l = smem + kOffB4l;
-    float *V = (float *)(smem + kOffV), *G = (float *)(smem + kOffG), *A = (float *)(smem + kOffA);
-    float *bet = (float *)(smem + kOffBeta);
-    uint64_t *bar = (uint64_t *)(smem + kOffBar);
+    uint64_t *bars = (uint64_t *)(smem + kOffBar);
     uint32_t *tbase = (uint32_t *)(smem + kOffTmem);
-    const int tid = threadIdx.x, w = tid >> 5, l = tid & 31;
-    const int quad = w & 3, half = w >> 2;
-    const int j = 32 * quad + l;                           // tensor-memory lane = value column
+    const int tid = threadIdx.x, w = tid >> 5;
     if (w == 0) {
         tc::tmem_alloc(tbase, kCols);
         tc::tmem_relinquish();
     }
     if (tid == 0) {
-        mbar_init(bar, 1);
+        mbar_init(&bars[kReady], kGroup);
+        mbar_init(&bars[kFull1], kGroup);
+        mbar_init(&bars[kP0], 1);
+        mbar_init(&bars[kP1], 1);
+        mbar_init(&bars[kWready], kGroup);
+        mbar_init(&bars[kFull2], kGroup);
+        mbar_init(&bars[kP2], 1);
+        mbar_init(&bars[kDrain], 1);
         mbar_init_fence();
     }
     tc::fence_before();
@@ -135,280 +550,18 @@ __global__ void __launch_bounds__(kThreads, 1) prefill_kernel(Args a) {
     griddep_wait();
     griddep_launch();
     const uint32_t tm = *tbase;                            // lane 0, first column
-    const uint32_t tl = tm + ((uint32_t)(32 * quad) << 16);   // this warp's lanes
-    uint32_t parity = 0;
-    bool alive = true;
-    const int grp = a.Hv / a.Hk;
-    // a CTA-wide bounded wait on the commit barrier; false if any thread gave up
-    const auto wait_mma = [&]() {
-        const bool ok = mbar_wait(bar, parity, pipe::kWaitCycles);
-        parity ^= 1u;
-        const bool stalled = __syncthreads_or(!ok);
-        tc::fence_after();
-        return !stalled;
-    };
-    // This thread's share of a chunk's operands, loaded one chunk ahead (their
-    // global-memory latency overlaps the previous chunk's tensor-core work):
-    // key channels 4 cq .. 4 cq + 3 at tokens 4 tq .. 4 tq + 3 of k, q, v (one
-    // 16-byte load each); threads 0..127 the chunk's gates of channel ci,
-    // threads 128..159 one beta each. Missing tokens of a ragged tail are the
-    // identity step (gate 1, beta 0, zero k, q, v).
-    const int ci = tid & 127, cq = tid & 31, tq = tid >> 5;
-    float4 kv[4], qv[4], vv[4];
-    float dg[C], bt = 0.f;
-    const auto fetch = [&](int it, int c0) {
-        const int fb = it / a.Hv, fh = it - fb * a.Hv, fhk = fh / grp, fn = min(C, a.T - c0);
-#pragma unroll
-        for (int m = 0; m < 4; m++) {
-            const int t = 4 * tq + m;
-            kv[m] = qv[m] = vv[m] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (t < fn) {
-                const size_t tok = (size_t)fb * a.T + c0 + t;
-                kv[m] = *(const float4 *)&a.k[(tok * a.Hk + fhk) * 128 + 4 * cq];
-                qv[m] = *(const float4 *)&a.q[(tok * a.Hk + fhk) * 128 + 4 * cq];
-                vv[m] = *(const float4 *)&a.v[(tok * a.Hv + fh) * 128 + 4 * cq];
-            }
-        }
-        if (tid < 128) {
-#pragma unroll
-            for (int t = 0; t < C; t++) {
-                const size_t tok = (size_t)fb * a.T + c0 + t;
-                float dv = 1.f;
-                if (t < fn) dv = a.gate_per_row ? a.gate[(tok * a.Hv + fh) * 128 + ci] : a.gate[tok * a.Hv + fh];
-                dg[t] = dv;
-            }
-        } else if (tid < 128 + C) {
-            const int t = tid - 128;
-            bt = t < fn ? a.beta[((size_t)fb * a.T + c0 + t) * a.Hv + fh] : 0.f;
-        }
-    };
-    // One chunk's cumulative gates g_t per key channel (multiplied in token
-    // order), beta, V and the split operands [K~ ; Q~] and K^, from the fetched
-    // registers, four consecutive K elements per store. K_bar^T, P2's operand,
-    // stays in kb until put_kbar (the previous chunk's P2 may still read it).
-    float kb[4][4];                                        // K_bar^T: [channel][token]
-    const auto prep = [&]() {
-        if (tid < 128) {
-            float g = 1.f;
-#pragma unroll
-            for (int t = 0; t < C; t++) {
-                g = fmaxf(g * dg[t], 1e-30f);             // keeps K / g finite
-                G[t * 128 + tid] = g;
-            }
-        } else if (tid < 128 + C) {
-            bet[tid - 128] = bt;
-        }
-        __syncthreads();
-        const int c4 = 4 * cq;
-        const float4 gC = *(const float4 *)&G[(C - 1) * 128 + c4];
-#pragma unroll
-        for (int m = 0; m < 4; m++) {
-            const int t = 4 * tq + m;
-            const float4 g = *(const float4 *)&G[t * 128 + c4];
-            const float4 rg = make_float4(__fdividef(1.0f, g.x), __fdividef(1.0f, g.y),   // within 2 ulp
-                                          __fdividef(1.0f, g.z), __fdividef(1.0f, g.w));
-            *(float4 *)&V[t * 128 + c4] = vv[m];
-            put_split4(B1h, B1l, core_off(t, c4, kSbo128), mul4(g, kv[m]));        // K~
-            put_split4(B1h, B1l, core_off(C + t, c4, kSbo128), mul4(g, qv[m]));    // Q~
-            put_split4(B3h, B3l, core_off(t, c4, kSbo128), mul4(kv[m], rg));       // K^
-            kb[0][m] = kv[m].x * (gC.x * rg.x);
-            kb[1][m] = kv[m].y * (gC.y * rg.y);
-            kb[2][m] = kv[m].z * (gC.z * rg.z);
-            kb[3][m] = kv[m].w * (gC.w * rg.w);
-        }
-    };
-    const auto put_kbar = [&]() {
-#pragma unroll
-        for (int e = 0; e < 4; e++)
-            put_split4(B2h, B2l, core_off(4 * cq + e, 4 * tq, kSbo32),
-                       make_float4(kb[e][0], kb[e][1], kb[e][2], kb[e][3]));
-    };
-    // This CTA's chunks in order: (item, first token); fi, fc is the chunk
-    // whose inputs the registers hold.
-    int fi = blockIdx.x, fc = 0;
-    const auto advance = [&]() {
-        fc += C;
-        if (fc >= a.T) {
-            fi += gridDim.x;
-            fc = 0;
-        }
-    };
-    // Prologue: the first chunk prepared, the second fetched.
-    if (fi < a.items) {
-        fetch(fi, fc);
-        prep();
-        put_kbar();
-        advance();
-        if (fi < a.items) fetch(fi, fc);
+    bool ok = true;
+    if (w < 8) {
+        tc::regs_inc<kRegsChain>();
+        ok = chain(a, smem, bars, tm);
+    } else if (w < 16) {
+        ok = produce(a, smem, bars);
+    } else {
+        tc::regs_dec<kRegsIssue>();
+        if (tid == 2 * kGroup) ok = issue_mma(a, smem, bars, tm);
     }
-    for (int item = blockIdx.x; alive && item < a.items; item += gridDim.x) {
-        const int b = item / a.Hv, h = item - b * a.Hv;
-        float *Sg = a.states + (size_t)item * kN;
-        // S^T into tensor memory: this thread's lane j, the 64 key rows of its half.
-        for (int c = 0; c < 2; c++) {
-            const int i0 = 64 * half + 32 * c;
-            float sv[32], hi[32], lo[32];
-#pragma unroll
-            for (int e = 0; e < 32; e++) {
-                sv[e] = Sg[(size_t)(i0 + e) * 128 + j];
-                tc::split_tf32(sv[e], hi[e], lo[e]);
-            }
-            tc::st32(tl + kColS + i0, sv);
-            tc::st32(tl + kColSh + i0, hi);
-            tc::st32(tl + kColSl + i0, lo);
-        }
-        tc::wait_st();
-        for (int t0 = 0; alive && t0 < a.T; t0 += C) {
-            const int n = min(C, a.T - t0);               // tokens in this chunk (ragged tail)
-            fence_async_smem();                           // this chunk's operands visible to the tensor cores
-            tc::fence_before();
-            __syncthreads();                              // the previous chunk is done with every buffer
-            // P0: [K~ ; Q~] K^T into columns [448, 480); P1: [K~ S_0 ; Q~ S_0]^T into [384, 448).
-            if (tid == 0) {
-                tc::fence_after();
-#pragma unroll 1
-                for (int s = 0; s < 16; s++) {
-                    const uint64_t ah = tc::sdesc(B1h + 2 * kLbo * s, kLbo, kSbo128), al = tc::sdesc(B1l + 2 * kLbo * s, kLbo, kSbo128);
-                    const uint64_t kh = tc::sdesc(B3h + 2 * kLbo * s, kLbo, kSbo128), kl = tc::sdesc(B3l + 2 * kLbo * s, kLbo, kSbo128);
-                    const uint32_t acc = s > 0 ? 1u : 0u;
-                    tc::mma_tf32_ss(tm + kColP0, ah, kh, kIdescP0, acc);
-                    tc::mma_tf32_ss(tm + kColP0, ah, kl, kIdescP0, 1u);
-                    tc::mma_tf32_ss(tm + kColP0, al, kh, kIdescP0, 1u);
-                    tc::mma_tf32_ts(tm + kColX, tm + kColSh + 8 * s, ah, kIdescP1, acc);
-                    tc::mma_tf32_ts(tm + kColX, tm + kColSh + 8 * s, al, kIdescP1, 1u);
-                    tc::mma_tf32_ts(tm + kColX, tm + kColSl + 8 * s, ah, kIdescP1, 1u);
-                }
-                tc::commit(bar);
-            }
-            __syncwarp();
-            if (!wait_mma()) {
-                alive = false;
-                break;
-            }
-            // A = strict lower of diag(beta) K~ K^T (row t = lane t), stored
-            // transposed (a warp's store is one row of A^T: no bank conflicts), and
-            // Bm = lower (with diagonal) of Q~ K^T (row t = lane 32 + t), Bm split
-            // as an operand.
-            if (w < 2) {
-                float d[32];
-                tc::ld32(tl + kColP0, d);
-                if (w == 0) {
-                    const float bt = bet[l];
-#pragma unroll
-                    for (int s = 0; s < C; s++) A[s * C + l] = s < l ? bt * d[s] : 0.f;
-                } else {
-#pragma unroll
-                    for (int s = 0; s < C; s++) put_split(B4h, B4l, core_off(l, s, kSbo32), s <= l ? d[s] : 0.f);
-                    fence_async_smem();
-                }
-            }
-            __syncthreads();                              // A visible; P0's columns free for W
-            if (half == 0) {
-                // W = (I + A)^-1 diag(beta) (V - K~ S_0), value column j, by forward
-                // substitution in column order: once w_s is final it is taken out
-                // of every later row (independent updates, so the dependent chain
-                // is one fma per token).
-                float wv[32];
-                tc::ld32(tl + kColX, wv);
-#pragma unroll
-                for (int t = 0; t < C; t++) wv[t] = bet[t] * (V[t * 128 + j] - wv[t]);
-#pragma unroll
-                for (int s = 0; s < C - 1; s++) {
-                    const float ws = wv[s];
-#pragma unroll
-                    for (int t4 = (s + 1) / 4; t4 < C / 4; t4++) {    // row s of A^T, four at a time
-                        const float4 a4 = ((const float4 *)(A + s * C))[t4];
-                        const float av[4] = {a4.x, a4.y, a4.z, a4.w};
-#pragma unroll
-                        for (int e = 0; e < 4; e++)
-                            if (4 * t4 + e > s) wv[4 * t4 + e] = fmaf(-av[e], ws, wv[4 * t4 + e]);
-                    }
-                }
-                float hi[32], lo[32];
-#pragma unroll
-                for (int t = 0; t < C; t++) tc::split_tf32(wv[t], hi[t], lo[t]);
-                tc::st32(tl + kColWh, hi);
-                tc::st32(tl + kColWl, lo);
-            } else {
-                // S^T <- S^T diag(g_C): key row i scaled by its cumulative gate.
-#pragma unroll 1
-                for (int c = 0; c < 4; c++) {
-                    float sv[32];
-                    tc::ld32(tl + kColS + 32 * c, sv);
-#pragma unroll
-                    for (int e = 0; e < 32; e++) sv[e] *= G[(C - 1) * 128 + 32 * c + e];
-                    tc::st32(tl + kColS + 32 * c, sv);
-                }
-            }
-            tc::wait_st();
-            tc::fence_before();
-            __syncthreads();
-            // P2: S^T += W^T K_bar; P3: Y^T = (Q~ S_0)^T + W^T Bm^T.
-            if (tid == 0) {
-                tc::fence_after();
-#pragma unroll 1
-                for (int s = 0; s < 4; s++) {
-                    const uint64_t bh = tc::sdesc(B2h + 2 * kLbo * s, kLbo, kSbo32), bl = tc::sdesc(B2l + 2 * kLbo * s, kLbo, kSbo32);
-                    const uint64_t mh = tc::sdesc(B4h + 2 * kLbo * s, kLbo, kSbo32), ml = tc::sdesc(B4l + 2 * kLbo * s, kLbo, kSbo32);
-                    tc::mma_tf32_ts(tm + kColS, tm + kColWh + 8 * s, bh, kIdescP2, 1u);
-                    tc::mma_tf32_ts(tm + kColS, tm + kColWh + 8 * s, bl, kIdescP2, 1u);
-                    tc::mma_tf32_ts(tm + kColS, tm + kColWl + 8 * s, bh, kIdescP2, 1u);
-                    tc::mma_tf32_ts(tm + kColY, tm + kColWh + 8 * s, mh, kIdescP3, 1u);
-                    tc::mma_tf32_ts(tm + kColY, tm + kColWh + 8 * s, ml, kIdescP3, 1u);
-                    tc::mma_tf32_ts(tm + kColY, tm + kColWl + 8 * s, mh, kIdescP3, 1u);
-                }
-                tc::commit(bar);
-            }
-            __syncwarp();
-            // While P2 and P3 run: the next chunk's operands (this item's next
-            // chunk or the next item's first), and the inputs of the one after.
-            const bool more = fi < a.items;
-            if (more) {
-                prep();
-                advance();
-                if (fi < a.items) fetch(fi, fc);
-            }
-            if (!wait_mma()) {
-                alive = false;
-                break;
-            }
-            if (more) put_kbar();                         // P2 is done with K_bar^T
-            // Outputs: tokens 16 half .. 16 half + 15 of column j.
-            {
-                float yv[16];
-                tc::ld16(tl + kColY + 16 * half, yv);
-#pragma unroll
-                for (int e = 0; e < 16; e++) {
-                    const int t = 16 * half + e;
-                    if (t < n) a.y[(((size_t)b * a.T + t0 + t) * a.Hv + h) * 128 + j] = yv[e];
-                }
-            }
-            // Heads and rests of the new state for the next chunk's P1.
-            for (int c = 0; c < 2; c++) {
-                const int i0 = 64 * half + 32 * c;
-                float sv[32], hi[32], lo[32];
-                tc::ld32(tl + kColS + i0, sv);
-#pragma unroll
-                for (int e = 0; e < 32; e++) tc::split_tf32(sv[e], hi[e], lo[e]);
-                tc::st32(tl + kColSh + i0, hi);
-                tc::st32(tl + kColSl + i0, lo);
-            }
-            tc::wait_st();
-        }
-        if (!alive) break;
-        // The boundary state back to global memory.
-        for (int c = 0; c < 2; c++) {
-            const int i0 = 64 * half + 32 * c;
-            float sv[32];
-            tc::ld32(tl + kColS + i0, sv);
-#pragma unroll
-            for (int e = 0; e < 32; e++) Sg[(size_t)(i0 + e) * 128 + j] = sv[e];
-        }
-    }
-    if (!alive && tid == 0) {
-        raise_error(a.err, STEPQ_ERR_TIMEOUT);
-        mbar_wait(bar, parity ^ 1u, pipe::kWaitCycles);  // the stalled MMAs, once more with a bound
-    }
+    if (!ok) raise_error(a.err, STEPQ_ERR_TIMEOUT);
+    __syncwarp();
     tc::fence_before();
     __syncthreads();
     if (w == 0) {
@@ -434,9 +587,15 @@ stepq_status launch_prefill(const stepq_config *cfg, const float *q, const float
     static SmemOptIn opt;
     const stepq_status st = opt((const void *)pf::prefill_kernel, pf::kSmem);
     if (st != STEPQ_OK) return st;
+    // the register shares are taken from what the kernel is launched with
+    static const int regs = [] {
+        cudaFuncAttributes f{};
+        return cudaFuncGetAttributes(&f, (const void *)pf::prefill_kernel) == cudaSuccess ? f.numRegs : 0;
+    }();
+    if (regs < pf::kRegs) return STEPQ_ERR_CUDA;
     int grid = sm_count();
     if (grid > a.items) grid = a.items;
-    return launch_overlapped(pf::prefill_kernel, grid, kThreads, pf::kSmem, s, a);
+    return launch_overlapped(pf::prefill_kernel, grid, pf::kBlock, pf::kSmem, s, a);
 }
 
 }  // namespace stepq
