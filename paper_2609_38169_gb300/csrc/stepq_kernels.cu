@@ -27,13 +27,13 @@ namespace stepq {
 // apart, hit 8 different bank groups instead of 2.
 constexpr int kFitRed = 0;                                   // float [2][8][128]
 constexpr int kFitCol = kFitRed + 2 * 8 * 128 * 4;           // float [2][128]: c_j, 1 / c_j
-constexpr int kFitRow = kFitCol + 2 * 128 * 4;               // float [4][128]: w^2, w^-1/2, rho, r
-constexpr int kFitBits = kFitRow + 4 * 128 * 4;              // int [128] widths
+constexpr int kFitRow = kFitCol + 2 * 128 * 4;               // float [5][128]: w^2, w^-1/2, rho, r, 1 / r
+constexpr int kFitBits = kFitRow + 5 * 128 * 4;              // int [128] widths
 constexpr int kFitWarp = kFitBits + 128 * 4;                 // float [8]
 constexpr int kFitBytes = kFitWarp + 64;
 
 struct FitSmem {
-    float *red, *colC, *colG, *w2, *wis, *rho, *rr, *warp;
+    float *red, *colC, *colG, *w2, *wis, *rho, *rr, *rho1, *warp;
     int *rbits;
     __device__ __forceinline__ explicit FitSmem(uint8_t *s) {
         red = (float *)(s + kFitRed);
@@ -43,6 +43,7 @@ struct FitSmem {
         wis = w2 + 128;
         rho = w2 + 256;
         rr = w2 + 384;
+        rho1 = w2 + 512;
         rbits = (int *)(s + kFitBits);
         warp = (float *)(s + kFitWarp);
     }
@@ -115,62 +116,78 @@ __device__ __forceinline__ void ls_partials(const Lane &L, const FitSmem &S, con
     }
 }
 
-// Key-Row-Aware Dual-axis Fitting of the register tile x (Sec. 4.3, App. C.1):
+// Key-Row-Aware Dual-axis Fitting of the register tile x (Sec. 4.3, App. C.1), in two
+// parts: the row factors with the columns' maxima, and the column factors.
 // x[t][e] holds columns 16cg + 2e, 2e + 1 of row 16w + 4t + rs. msum[t]: sum_j
-// |X_ij| of the thread's rows; row widths come from S.rbits. On return S.rho and
-// S.rr hold the rows' reciprocal and stored row factors, S.colC the stored
-// (FP16-rounded) column factors and S.colG their reciprocals; a page (or null)
-// receives the FP16 r and c and must no longer be read. Returns whether a code may
-// exceed qmax with these scales (uniform over the CTA).
+// |X_ij| of the thread's rows; row widths come from S.rbits.
 //
 // Bound by instruction issue (about 60% of it fp32 arithmetic), so the passes run
 // on f32x2 column pairs, and the clamps, two min/max per code, only when the clip-free
 // start was capped, the state holds a non-finite value or (last pass and final
 // codes) some max_i |X'_ij| mu_i / c_j reaches 1 + 1/(2 qmax).
-__device__ __forceinline__ bool fit_scales(const Lane &L, const FitSmem &S, const uint64_t (&x)[4][8],
-                                           const float (&msum)[4], int unit_rows, uint8_t *page,
-                                           int fit_iters) {
-    // Row factors r_i = m_i^(1/2) w_i^(-1/2), and the clip-free column start
-    // c0_j = max_i fp32(fp32(|X_ij| rho_i) mu_i), mu_i = 1 / qmax_i.
-    bool wild = false;                                       // a non-finite row sum
+
+// Row factors r_i = m_i^(1/2) w_i^(-1/2) into S.rr (and the page, or null, which must no
+// longer be read), rho_i = 1 / (r_i zs_i) into S.rho (0 for pivot rows). Thread tid < 128
+// returns column tid's clip-free start c0_j = max_i fp32(fp32(|X_ij| rho_i) mu_i),
+// mu_i = 1 / qmax_i; ANY leaves out the widths (mu_i = zs_i = 1, rho_i into S.rho1): a head
+// of one width has that maximum and those rho_i times a power of two, and the start is
+// rounded once more by mu (rounding keeps the order). `wild`: a non-finite row sum.
+template <bool ANY>
+__device__ __forceinline__ float fit_rows(const Lane &L, const FitSmem &S, const uint64_t (&x)[4][8],
+                                          const float (&msum)[4], int unit_rows, uint8_t *page, bool &wild) {
+    wild = false;
     float acc[16];
 #pragma unroll
     for (int j = 0; j < 16; j++) acc[j] = 0.f;
 #pragma unroll
     for (int t = 0; t < 4; t++) {
         const int i = L.row(t), bits = S.rbits[i];
-        float rf = 0.f, rho = 0.f, mu = 0.f;
+        float rf = 0.f, rho = 0.f, zs = 1.f, mu = 0.f;
         if (bits != kPivot) {
             const float m = msum[t] * (1.0f / 128.0f);
             rf = __half2float(__float2half_rn(
                 fminf(fmaxf(__fmul_rn(sqrtf(m), S.wis[i]), kF16Min), kF16Max)));
-            const float zs = unit_rows ? (float)(1 << (8 - bits)) : 1.0f;
+            if (!ANY) {
+                zs = unit_rows ? (float)(1 << (8 - bits)) : 1.0f;
+                mu = __frcp_rn((float)qmax_of(bits));
+            }
             rho = __frcp_rn(rf * zs);
-            mu = __frcp_rn((float)qmax_of(bits));
         }
         wild = wild || !(msum[t] <= 3.4028235e38f);
         if (L.cg == 0) {
             S.rr[i] = rf;
-            S.rho[i] = rho;
+            (ANY ? S.rho1 : S.rho)[i] = rho;
             if (page) ((uint16_t *)page)[i] = f16_bits(rf);
         }
         const uint64_t rho2 = f2s(rho), mu2 = f2s(mu);
 #pragma unroll
         for (int e = 0; e < 8; e++) {
-            const uint64_t z = fmul2(fmul2(x[t][e], rho2), mu2);
+            uint64_t z = fmul2(x[t][e], rho2);
+            if (!ANY) z = fmul2(z, mu2);
             acc[2 * e] = fmaxf(acc[2 * e], fabsf(f2lo(z)));
             acc[2 * e + 1] = fmaxf(acc[2 * e + 1], fabsf(f2hi(z)));
         }
     }
     columns_to_red<true>(L, acc, S.red);
     __syncthreads();
-    // Threads 0..127 own one column each: its start c0, its current iterate.
     const int cp = cpos(L.tid & 127);
-    float cm = 0.f, cc = 0.f;
+    float cm = 0.f;
     if (L.tid < 128) {
         cm = S.red[cp];
 #pragma unroll
         for (int wv = 1; wv < 8; wv++) cm = fmaxf(cm, S.red[wv * 128 + cp]);
+    }
+    return cm;
+}
+
+// Column factors from the starts cm (thread tid < 128: column tid): S.colC the stored
+// (FP16-rounded) ones, S.colG their reciprocals, the page (or null) the FP16 c. Returns
+// whether a code may exceed qmax with these scales (uniform over the CTA).
+__device__ __forceinline__ bool fit_columns(const Lane &L, const FitSmem &S, const uint64_t (&x)[4][8], float cm,
+                                            bool wild, int unit_rows, uint8_t *page, int fit_iters) {
+    const int cp = cpos(L.tid & 127);
+    float acc[16], cc = 0.f;
+    if (L.tid < 128) {
         wild = wild || cm > kF16Max;                         // start capped: codes may clip
         cc = fminf(fmaxf(cm, kF16Min), kF16Max);
         S.colG[cp] = __frcp_rn(cc);
@@ -351,7 +368,7 @@ struct PoolArgs {
 // refilled with the next item's state (16-byte cp.async, swizzled as cgroup), and the
 // page leaves by a bulk store. One CTA per item with plain loads exposed their
 // latency (stalled on it 18% of the time at 24% occupancy): 4096 heads at 6 bits
-// took 143 us, 112 us now (47 us at the copy rate of HBM).
+// took 143 us, 110 us now (47 us at the copy rate of HBM).
 constexpr int kQTile = 0;                                    // float [128][128], 16-byte groups swizzled
 constexpr int kQPage = kN * 4;
 constexpr int kQFit = kQPage + (int)kMaxHeadBytes;
@@ -435,7 +452,9 @@ __global__ void __launch_bounds__(kThreads, 2) quantize_kernel(PoolArgs a) {
             start(next);
             fetch(next);
         }
-        const bool clip = fit_scales(L, S, x, msum, 1, page, a.fit_iters);
+        bool wild;
+        const float cm = fit_rows<false>(L, S, x, msum, 1, page, wild);
+        const bool clip = fit_columns(L, S, x, cm, wild, 1, page, a.fit_iters);
         pack_page(L, S, page, roff, x, clip);
         fence_async_smem();
         __syncthreads();
@@ -534,12 +553,26 @@ __device__ __forceinline__ void distortion_of(const Lane &L, const FitSmem &S, c
                                               const float (&msum)[4], const uint8_t *piv, const FitCands &a,
                                               const Add &add) {
     const int K1 = a.n_cand + 1;
+    // The row factors and the columns' maxima serve every candidate (formed anew for each
+    // of three, the four-layer model's calibration took 12.0 ms; 11.0 ms now).
+    if (L.tid < 128) S.rbits[L.tid] = piv && piv[L.tid] ? kPivot : a.cands[0];
+    __syncthreads();
+    bool wild;
+    const float top = fit_rows<true>(L, S, x, msum, a.unit_rows, nullptr, wild);
     for (int k = 0; k < K1; k++) {
         const bool fp16_col = (k == a.n_cand);
-        if (L.tid < 128) S.rbits[L.tid] = fp16_col || (piv && piv[L.tid]) ? kPivot : a.cands[k];
+        const int b = fp16_col ? kPivot : a.cands[k];
+        const float step = fp16_col || !a.unit_rows ? 1.f : 1.0f / (float)(1 << (8 - b));
+        if (L.tid < 128) {
+            S.rbits[L.tid] = piv && piv[L.tid] ? kPivot : b;
+            S.rho[L.tid] = S.rho1[L.tid] * step;              // 0 stays 0 for a pivot row
+        }
         __syncthreads();
         bool clip = false;
-        if (!fp16_col) clip = fit_scales(L, S, x, msum, a.unit_rows, nullptr, a.fit_iters);
+        if (!fp16_col) {
+            const float cm = __fmul_rn(top * step, __frcp_rn((float)qmax_of(b)));
+            clip = fit_columns(L, S, x, cm, wild, a.unit_rows, nullptr, a.fit_iters);
+        }
         float head_err = 0.f;
 #pragma unroll
         for (int t = 0; t < 4; t++) {
