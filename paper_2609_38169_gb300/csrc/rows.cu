@@ -8,9 +8,9 @@
 // segment of the row. A thread holds 8 slot pairs x 4 columns as packed f32x2
 // registers: per-row constants of a pair are adjacent in shared memory (one
 // 128-bit load serves two pairs), column constants are duplicated pairs kept
-// in registers. Widths are handled with runtime shifts and masks (one funnel
-// shift per row segment), which keeps the unrolled code small; FP16 pivot rows
-// take an out-of-line path.
+// in registers. Widths are handled with runtime shifts and masks, formed once
+// for four rows (kQuad), which keeps the unrolled code small; rows of mixed
+// quads and FP16 pivot rows take an out-of-line path.
 //
 // Per row i the tile holds Z with X_ij = a_i Z_ij: a_i = d_i r_i zs_i and
 // Z = c_j q_ij for an integer row (zs_i = 2^(8 - b_i), the normalised codebook
@@ -128,44 +128,20 @@ __device__ __forceinline__ uint64_t clamp2p(uint64_t v, uint64_t lim) {
     return f2(fminf(fmaxf(f2lo(v), -a), a), fminf(fmaxf(f2hi(v), -b), b));
 }
 
-// The lane's 4b-bit code segment of a row of width b (columns 4l..4l+3),
-// right-aligned. The second word may lie past the row; it stays inside the
-// stage and its bits beyond the segment are masked off by the callers.
-__device__ __forceinline__ uint32_t lane_segment(const uint8_t *row, int b, int l) {
-    const uint32_t *wp = (const uint32_t *)row;
-    const int bit = 4 * l * b;
-    return __funnelshift_r(wp[bit >> 5], wp[(bit >> 5) + 1], bit & 31);
+// The lane's 4b-bit code segment (columns 4l..4l+3) of a row of width b, right-aligned;
+// wp is the word that it begins in. The second word may lie past the row; it stays inside
+// the stage, and its bits beyond the segment are masked off by the callers.
+__device__ __forceinline__ uint32_t lane_segment(const uint32_t *wp, int b, int l) {
+    return __funnelshift_r(wp[0], wp[1], 4 * l * b);
 }
-
-// Write the lane's 4b-bit segment v (b in {2, 4, 6, 8}) into the row: b/2
-// bytes from byte l b/2, as byte stores under warp-uniform conditions (no
-// branches; the lanes never share a byte).
-__device__ __forceinline__ void store_segment(uint8_t *row, int b, int l, uint32_t v) {
-    uint8_t *p = row + ((l * b) >> 1);
-    p[0] = (uint8_t)v;
-    if (b >= 4) p[1] = (uint8_t)(v >> 8);
-    if (b >= 6) p[2] = (uint8_t)(v >> 16);
-    if (b >= 8) p[3] = (uint8_t)(v >> 24);
+__device__ __forceinline__ const uint32_t *lane_word(const uint8_t *row, int b, int l) {
+    return (const uint32_t *)row + ((l * b) >> 3);
 }
 
 // Sum over the 4 codes of a lane segment of (0x4B400000 << k b): what the
 // packing adds besides the codes.
 __device__ __forceinline__ uint32_t pack_bias4(int b) {
     return kMagicBits + (kMagicBits << b) + (kMagicBits << (2 * b)) + (kMagicBits << (3 * b));
-}
-
-// FP16 pivot rows (rare): kept out of line so the unrolled tile loops stay small.
-__device__ __noinline__ float4 pivot_values(const uint8_t *row, int l) {
-    const uint2 p = ((const uint2 *)row)[l];
-    return make_float4(f16_val((uint16_t)(p.x & 0xFFFFu)), f16_val((uint16_t)(p.x >> 16)),
-                       f16_val((uint16_t)(p.y & 0xFFFFu)), f16_val((uint16_t)(p.y >> 16)));
-}
-__device__ __noinline__ void store_pivot(uint8_t *row, int l, float a, float4 z) {
-    const uint32_t w0 = (uint32_t)f16_bits(f16_round_sat(a * z.x)) |
-                        ((uint32_t)f16_bits(f16_round_sat(a * z.y)) << 16);
-    const uint32_t w1 = (uint32_t)f16_bits(f16_round_sat(a * z.z)) |
-                        ((uint32_t)f16_bits(f16_round_sat(a * z.w)) << 16);
-    ((uint2 *)row)[l] = make_uint2(w0, w1);
 }
 
 // ------------------------------------------------------------------ decode
@@ -216,85 +192,148 @@ __device__ __forceinline__ void issue(const DecodeArgs &a, const Smem &S, int h,
     }
 }
 
-// Z of row pair m (columns 4l..4l+3): c_j q_ij (exact) for integer rows, the
-// FP16 value for pivot rows.
-__device__ __forceinline__ void load_pair(const T &t, const Smem &S, const uint8_t *page, int m,
-                                          const uint64_t (&cd)[4], uint64_t (&x)[4]) {
-    const uint4 inf = *(const uint4 *)&S.rInfo[t.row(2 * m)];
-    const int b0 = (int)((inf.x >> 16) & 0xFFu), b1 = (int)((inf.z >> 16) & 0xFFu);
-    const uint8_t *r0 = page + (inf.x & 0xFFFFu), *r1 = page + (inf.z & 0xFFFFu);
-    if (b0 != kPivot && b1 != kPivot) {                  // two integer rows: paired arithmetic
-        const uint32_t s0 = lane_segment(r0, b0, t.l), s1 = lane_segment(r1, b1, t.l);
-        const uint32_t k0 = (1u << b0) - 1u, k1 = (1u << b1) - 1u;
-        const uint64_t off = row_pair(S.rOff, t, m);
-#pragma unroll
-        for (int c = 0; c < 4; c++)
-            x[c] = fmul2(fadd2(u2pair(and_or(s0 >> (c * b0), k0, kMagicBits), and_or(s1 >> (c * b1), k1, kMagicBits)),
-                               off),
-                         cd[c]);
-        return;
+// Slots are read and written in quads of four. Rows are stored by decreasing width, so all
+// but a few quads of a head hold integer rows of one width, each where the one before ends
+// (kQuad): addresses, shifts and masks are formed once for 16 codes. The width stays a
+// run-time value: with a body per width (a fifth fewer instructions again) the warps no
+// longer ran the same code, and waiting for it (no instruction: 0.5 -> 1.6 to 2.0 cycles
+// an issue) cost more than it gave. 256 sequences of 32 heads at 4 bits: 199 us so, 195 us
+// with every shift formed per row pair, 179 us here; four layers of 128 sequences at 6 bits:
+// 438, 417 and 366 us. The other quads, those that hold a change of width or FP16 rows, go
+// row by row through functions out of line, which keeps the code that every warp runs small.
+constexpr uint32_t kQuad = 1u << 31;                   // in the info of a quad's slots
+
+__device__ __noinline__ float4 row_values(const uint8_t *row, int b, int l, float4 c) {
+    if (b == kPivot) {
+        const uint2 p = ((const uint2 *)row)[l];
+        return make_float4(f16_val((uint16_t)(p.x & 0xFFFFu)), f16_val((uint16_t)(p.x >> 16)),
+                           f16_val((uint16_t)(p.y & 0xFFFFu)), f16_val((uint16_t)(p.y >> 16)));
     }
-    float v[2][4];
-#pragma unroll
-    for (int h = 0; h < 2; h++) {
-        const int b = h ? b1 : b0;
-        const uint8_t *row = h ? r1 : r0;
-        if (b == kPivot) {
-            const float4 p = pivot_values(row, t.l);
-            v[h][0] = p.x;
-            v[h][1] = p.y;
-            v[h][2] = p.z;
-            v[h][3] = p.w;
-        } else {
-            const uint32_t s = lane_segment(row, b, t.l), k = (1u << b) - 1u;
-            const float off = S.rOff[t.row(2 * m + h)];
-#pragma unroll
-            for (int c = 0; c < 4; c++)
-                v[h][c] = __fmul_rn(__uint_as_float(and_or(s >> (c * b), k, kMagicBits)) + off,
-                                    f2lo(cd[c]));
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < 4; c++) x[c] = f2(v[0][c], v[1][c]);
+    const uint32_t s = lane_segment(lane_word(row, b, l), b, l), k = (1u << b) - 1u;
+    const float off = -(kMagic + (float)(1 << (b - 1)));
+    return make_float4(__fmul_rn(__uint_as_float(and_or(s, k, kMagicBits)) + off, c.x),
+                       __fmul_rn(__uint_as_float(and_or(s >> b, k, kMagicBits)) + off, c.y),
+                       __fmul_rn(__uint_as_float(and_or(s >> (2 * b), k, kMagicBits)) + off, c.z),
+                       __fmul_rn(__uint_as_float(and_or(s >> (3 * b), k, kMagicBits)) + off, c.w));
 }
 
-// Final codes of row pair m: q = rne(X' / c_j) (clamped to +-qmax when CLIP),
-// or fp16(a Z) for a pivot row, written into the page.
-template <bool CLIP>
-__device__ __forceinline__ void store_pair(const T &t, const Smem &S, uint8_t *page, int m,
-                                           const uint64_t (&x)[4], const uint64_t (&gd)[4]) {
-    const uint4 inf = *(const uint4 *)&S.rInfo[t.row(2 * m)];
-    const int b0 = (int)((inf.x >> 16) & 0xFFu), b1 = (int)((inf.z >> 16) & 0xFFu);
-    uint8_t *r0 = page + (inf.x & 0xFFFFu), *r1 = page + (inf.z & 0xFFFFu);
-    const uint64_t mb = row_pair(S.rMb, t, m);
-    uint64_t lo = 0, hi = 0;
-    if (CLIP) {
-        const uint64_t qm = row_pair(S.rQm, t, m);
-        lo = f2(f2lo(mb) - f2lo(qm), f2hi(mb) - f2hi(qm));
-        hi = f2(f2lo(mb) + f2lo(qm), f2hi(mb) + f2hi(qm));
+// The codes of slot info.x (width b, pack bias info.y), or fp16(a Z) for a pivot row.
+__device__ __noinline__ void store_row(uint8_t *page, uint2 info, int l, bool clip, float a, float4 z, float4 g) {
+    uint8_t *row = page + (info.x & 0xFFFFu);
+    const int b = (int)((info.x >> 16) & 0xFFu);
+    if (b == kPivot) {
+        const uint32_t w0 = (uint32_t)f16_bits(f16_round_sat(a * z.x)) |
+                            ((uint32_t)f16_bits(f16_round_sat(a * z.y)) << 16);
+        const uint32_t w1 = (uint32_t)f16_bits(f16_round_sat(a * z.z)) |
+                            ((uint32_t)f16_bits(f16_round_sat(a * z.w)) << 16);
+        ((uint2 *)row)[l] = make_uint2(w0, w1);
+        return;
     }
-    uint32_t f[2][4];
+    const float mb = kMagic + (float)(1 << (b - 1));
+    float u[4] = {__fmaf_rn(z.x, g.x, mb), __fmaf_rn(z.y, g.y, mb), __fmaf_rn(z.z, g.z, mb), __fmaf_rn(z.w, g.w, mb)};
+    uint32_t v = 0;
 #pragma unroll
-    for (int c = 0; c < 4; c++) {
-        // one rounding of the exact product, then the clamp on the biased code
-        uint64_t uu = ffma2(x[c], gd[c], mb);           // bits: 0x4B400000 | (q + 2^(b-1))
-        if (CLIP) uu = clamp2r(uu, lo, hi);
-        f[0][c] = (uint32_t)uu;
-        f[1][c] = (uint32_t)(uu >> 32);
+    for (int c = 3; c >= 0; c--) {
+        if (clip) u[c] = fminf(fmaxf(u[c], kMagic + 1.f), kMagic + (float)((1 << b) - 1));
+        v = (v << b) + __float_as_uint(u[c]);
     }
+    v -= info.y;
+    uint8_t *p = row + ((l * b) >> 1);                   // the lanes never share a byte
+    p[0] = (uint8_t)v;
+    if (b >= 4) p[1] = (uint8_t)(v >> 8);
+    if (b >= 6) p[2] = (uint8_t)(v >> 16);
+    if (b >= 8) p[3] = (uint8_t)(v >> 24);
+}
+
+// Z of the warp's slots 4p..4p+3 (columns 4l..4l+3): c_j q_ij (exact) for integer rows, the
+// FP16 value for pivot rows.
+__device__ __forceinline__ void load_quad(const T &t, const Smem &S, const uint8_t *page, int p,
+                                          const uint64_t (&cd)[4], uint64_t (&xa)[4], uint64_t (&xb)[4]) {
+    const uint32_t inf = S.rInfo[t.row(4 * p)].x;
+    if (inf & kQuad) {
+        const int b = (int)((inf >> 16) & 0xFFu);
+        const uint32_t *wp = lane_word(page + (inf & 0xFFFFu), b, t.l);
+        const uint32_t k = (1u << b) - 1u;
+        const uint64_t off = row_pair(S.rOff, t, 2 * p);   // one width: a pair of equals
+        uint32_t s[4];
 #pragma unroll
-    for (int h = 0; h < 2; h++) {
-        const int b = h ? b1 : b0;
-        uint8_t *row = h ? r1 : r0;
-        if (b == kPivot) {
-            store_pivot(row, t.l, S.rA[t.row(2 * m + h)],
-                        make_float4(h ? f2hi(x[0]) : f2lo(x[0]), h ? f2hi(x[1]) : f2lo(x[1]),
-                                    h ? f2hi(x[2]) : f2lo(x[2]), h ? f2hi(x[3]) : f2lo(x[3])));
-        } else {
-            const uint32_t K = h ? inf.w : inf.y;
-            const uint32_t v = f[h][0] + (f[h][1] << b) + (f[h][2] << (2 * b)) + (f[h][3] << (3 * b)) - K;
-            store_segment(row, b, t.l, v);
+        for (int r = 0; r < 4; r++) s[r] = lane_segment(wp + 4 * b * r, b, t.l);
+#pragma unroll
+        for (int c = 0; c < 4; c++) {
+            xa[c] = fmul2(fadd2(u2pair(and_or(s[0] >> (c * b), k, kMagicBits), and_or(s[1] >> (c * b), k, kMagicBits)),
+                                off), cd[c]);
+            xb[c] = fmul2(fadd2(u2pair(and_or(s[2] >> (c * b), k, kMagicBits), and_or(s[3] >> (c * b), k, kMagicBits)),
+                                off), cd[c]);
         }
+        return;
+    }
+    const float4 cc = make_float4(f2lo(cd[0]), f2lo(cd[1]), f2lo(cd[2]), f2lo(cd[3]));
+    float4 v[4];
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        const uint32_t i = S.rInfo[t.row(4 * p + r)].x;
+        v[r] = row_values(page + (i & 0xFFFFu), (int)((i >> 16) & 0xFFu), t.l, cc);
+    }
+    xa[0] = f2(v[0].x, v[1].x); xa[1] = f2(v[0].y, v[1].y); xa[2] = f2(v[0].z, v[1].z); xa[3] = f2(v[0].w, v[1].w);
+    xb[0] = f2(v[2].x, v[3].x); xb[1] = f2(v[2].y, v[3].y); xb[2] = f2(v[2].z, v[3].z); xb[3] = f2(v[2].w, v[3].w);
+}
+
+// Final codes of slots 4p..4p+3: q = rne(X' / c_j) (clamped to +-qmax when CLIP), or
+// fp16(a Z) for a pivot row, written into the page.
+template <bool CLIP>
+__device__ __forceinline__ void store_quad(const T &t, const Smem &S, uint8_t *page, int p,
+                                           const uint64_t (&xa)[4], const uint64_t (&xb)[4], const uint64_t (&gd)[4]) {
+    const uint2 inf = S.rInfo[t.row(4 * p)];
+    if (inf.x & kQuad) {
+        const int b = (int)((inf.x >> 16) & 0xFFu);
+        const uint32_t m = 1u << b;
+        const uint64_t mb = row_pair(S.rMb, t, 2 * p), lo = f2s(kMagic + 1.f),   // mb -+ qmax
+                       hi = f2s(__uint_as_float(kMagicBits + m - 1u));
+        uint32_t v[4] = {0, 0, 0, 0};
+#pragma unroll
+        for (int c = 3; c >= 0; c--) {
+            // one rounding of the exact product, then the clamp on the biased code;
+            // bits: 0x4B400000 | (q + 2^(b-1))
+            uint64_t ua = ffma2(xa[c], gd[c], mb), ub = ffma2(xb[c], gd[c], mb);
+            if (CLIP) {
+                ua = clamp2r(ua, lo, hi);
+                ub = clamp2r(ub, lo, hi);
+            }
+            v[0] = v[0] * m + (uint32_t)ua;
+            v[1] = v[1] * m + (uint32_t)(ua >> 32);
+            v[2] = v[2] * m + (uint32_t)ub;
+            v[3] = v[3] * m + (uint32_t)(ub >> 32);
+        }
+        uint8_t *q = page + (inf.x & 0xFFFFu) + ((t.l * b) >> 1);
+#pragma unroll
+        for (int r = 0; r < 4; r++) v[r] -= inf.y;
+        if (b == 4) {
+#pragma unroll
+            for (int r = 0; r < 4; r++) *(uint16_t *)(q + 64 * r) = (uint16_t)v[r];
+        } else if (b == 8) {
+#pragma unroll
+            for (int r = 0; r < 4; r++) *(uint32_t *)(q + 128 * r) = v[r];
+        } else if (b == 6) {
+#pragma unroll
+            for (int r = 0; r < 4; r++) {
+                q[96 * r] = (uint8_t)v[r];
+                q[96 * r + 1] = (uint8_t)(v[r] >> 8);
+                q[96 * r + 2] = (uint8_t)(v[r] >> 16);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < 4; r++) q[32 * r] = (uint8_t)v[r];
+        }
+        return;
+    }
+    const float4 g = make_float4(f2lo(gd[0]), f2lo(gd[1]), f2lo(gd[2]), f2lo(gd[3]));
+#pragma unroll
+    for (int r = 0; r < 4; r++) {
+        const uint64_t(&x)[4] = r < 2 ? xa : xb;
+        const int sl = t.row(4 * p + r);
+        store_row(page, S.rInfo[sl], t.l, CLIP, S.rA[sl],
+                  r & 1 ? make_float4(f2hi(x[0]), f2hi(x[1]), f2hi(x[2]), f2hi(x[3]))
+                        : make_float4(f2lo(x[0]), f2lo(x[1]), f2lo(x[2]), f2lo(x[3])), g);
     }
 }
 
@@ -337,9 +376,10 @@ __device__ __forceinline__ bool decode_item(const T &t, const Smem &S, const Sta
                                             const Refill &refill) {
     uint16_t *page_r = (uint16_t *)st.page;
     uint16_t *page_c = (uint16_t *)(st.page + 256);
-    // Row constants of the warp's band (warp-local).
-    if (t.l < 16) {
-        const int sl = t.row(t.l);                         // stored slot; i = its key row
+    // Row constants of the warp's band (warp-local); both halves of the warp form and
+    // write them, so that the votes on the quads see whole warps.
+    {
+        const int sl = t.row(t.l & 15);                    // stored slot; i = its key row
         // The row table arrives with the page; a stage whose copies did not
         // complete still holds whatever it held, and the first CTA barrier ends
         // the item then. Offset and width are capped first, and the offset
@@ -349,8 +389,11 @@ __device__ __forceinline__ bool decode_item(const T &t, const Smem &S, const Sta
         const uint32_t raw = st.slot[sl];
         const uint32_t region = (uint32_t)((const uint8_t *)st.q - st.page);
         const uint32_t off = min(raw & 0xFFFFu, region) & ~31u, bw = min((raw >> 16) & 0xFFu, (uint32_t)kPivot);
-        const uint32_t info = off | (bw << 16) | (raw & 0xFF000000u);
-        const int b = (int)bw, i = (int)(info >> 24);
+        const int b = (int)bw, i = (int)(raw >> 24) & 127;
+        const uint32_t first = __shfl_sync(0xffffffffu, off | (bw << 16), t.l & ~3);
+        const bool fits = (off | (bw << 16)) == first + 16u * bw * (t.l & 3) && b != kPivot;
+        const uint32_t vote = __ballot_sync(0xffffffffu, fits) >> (t.l & ~3) & 15u;
+        const uint32_t info = off | (bw << 16) | ((uint32_t)i << 24) | (vote == 15u ? kQuad : 0u);
         const float dg = st.gate[i];
         float a = dg, mu = 0.f, qm = 0.f, mb = 0.f;
         uint32_t K = 0;
@@ -385,7 +428,7 @@ __device__ __forceinline__ bool decode_item(const T &t, const Smem &S, const Sta
         cd[2] = f2s(f16_val((uint16_t)(cb.y & 0xFFFFu)));
         cd[3] = f2s(f16_val((uint16_t)(cb.y >> 16)));
 #pragma unroll
-        for (int m = 0; m < 8; m++) load_pair(t, S, st.page, m, cd, x2[m]);
+        for (int p = 0; p < 4; p++) load_quad(t, S, st.page, p, cd, x2[2 * p], x2[2 * p + 1]);
     }
     float rs[16];
     if constexpr (MODE == kWriteback) {
@@ -490,7 +533,7 @@ __device__ __forceinline__ bool decode_item(const T &t, const Smem &S, const Sta
         const int sl = t.row(rr);
         if ((t.l & 1) == 0) {
             const uint32_t info = S.rInfo[sl].x;
-            const int b = (int)((info >> 16) & 0xFFu), i = (int)(info >> 24);
+            const int b = (int)((info >> 16) & 0xFFu), i = (int)(info >> 24) & 127;
             if (b == kPivot) {
                 S.rRho[sl] = 1.f;
                 S.rAl[sl] = 0.f;
@@ -595,10 +638,10 @@ __device__ __forceinline__ bool decode_item(const T &t, const Smem &S, const Sta
         col_dup(S.colG, t.l, gd);
         if (S.flags[2]) {
 #pragma unroll
-            for (int m = 0; m < 8; m++) store_pair<true>(t, S, st.page, m, x2[m], gd);
+            for (int p = 0; p < 4; p++) store_quad<true>(t, S, st.page, p, x2[2 * p], x2[2 * p + 1], gd);
         } else {
 #pragma unroll
-            for (int m = 0; m < 8; m++) store_pair<false>(t, S, st.page, m, x2[m], gd);
+            for (int p = 0; p < 4; p++) store_quad<false>(t, S, st.page, p, x2[2 * p], x2[2 * p + 1], gd);
         }
     }
     return true;
