@@ -133,10 +133,11 @@ void stepq_plan_destroy(stepq_plan *plan);
 /* ----------------------------------------------------------------- device path
  * Pool: device, pool_slots * slot_stride bytes, 256-byte aligned. Slot page s
  * starts at pool + s * slot_stride and holds every (layer, head) segment:
- *   integer head unit: r[128] fp16 | c[128] fp16 | codes in chunks: the 16
- *                      codes of band g (rows 16g..16g+15) in column j take 2b
- *                      bytes, chunk index ((j / 4) * 8 + g) * 4 + j % 4
- *   FP16 pivot head:   the same chunk order of fp16 values (32 bytes per chunk)
+ *   integer head unit: r[128] fp16 | c[128] fp16 | codes in streams of 8b bytes:
+ *                      the 64 codes of band g (rows 16g..16g+15) in columns
+ *                      4t..4t+3, column by column; 16-byte piece k of the stream
+ *                      lies at 512 + (t / 4) * 256b + 512k + 16 * (8 (t % 4) + g)
+ *   FP16 pivot head:   the same arrangement of fp16 values (b = 16, no r and c)
  *   row-unit head:     r[128] fp16 | c[128] fp16 | the rows, 16*b_i bytes each
  *                      (b_i = 16: fp16 row), stored by decreasing width, rows of
  *                      equal width in index order

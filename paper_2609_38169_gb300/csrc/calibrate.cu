@@ -42,12 +42,16 @@ struct Workspace {
         acc = (double *)take(U * K1 * sizeof(double));
         w = (float *)take(heads * kD * sizeof(float));
         pivot = take(U);
-        // About 16 observe CTAs per SM, within the size of n dense states of a layer
-        // (what the workspace of n sequences has always had room for).
+        // About 16 observe CTAs per SM, within the size of n dense states of a layer.
         const size_t most = std::max<size_t>(1, 32 * (size_t)n / cfg->n_layers);
         chunks = (int)std::min(most, (16 * 152 + heads - 1) / heads);
-        scratch = (double *)take(chunks > 1 ? chunks * heads * 2 * kD * sizeof(double) : 0);
-        if (chunks == 1) scratch = nullptr;
+        scratch = base && chunks > 1 ? (double *)(base + o) : nullptr;
+        // The size is part of the interface, in what is asked for and in what is refused:
+        // n slot ids, n dense states and n readouts of a layer, as when the replay went
+        // through memory.
+        take((size_t)n * sizeof(int32_t));
+        take((size_t)n * cfg->n_value_heads * kN * sizeof(float));
+        take((size_t)n * cfg->n_value_heads * kD * sizeof(float));
         bytes = o;
     }
 };

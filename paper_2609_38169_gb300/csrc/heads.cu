@@ -675,7 +675,7 @@ struct PoolArgs {
 // registers its shared-memory copy is refilled with the next item's state (16-byte
 // cp.async), so the loads run under the fit, and the page leaves by a bulk store.
 // (One CTA per item with plain loads was stalled on them half of the time: 106 us for
-// 4096 heads at 6 bits, 60 us now; 47 us at the copy rate of HBM.) The 16-byte
+// 4096 heads at 6 bits, 58 us now; 47 us at the copy rate of HBM.) The 16-byte
 // groups of a row are swizzled by its band, so that the 8 lanes of a quarter warp,
 // which read one column quad of 8 bands, hit 8 bank groups.
 constexpr int kPageMaxHead = 32768;
@@ -789,7 +789,7 @@ __device__ __forceinline__ void dequantize_item(const T &t, const uint8_t *page,
 // from the page in whole 512-byte requests; the dense rows, of which a warp holds 64
 // bytes each, meet in shared memory and leave as one 8 KB bulk store a band. (Staging
 // the page first and storing the 64-byte pieces took 98 us for 4096 heads at 6 bits,
-// direct reads with those stores 73 us, this form 53 us; 47 us at the copy rate of
+// direct reads with those stores 73 us, this form 51 us; 47 us at the copy rate of
 // HBM.)
 __global__ void __launch_bounds__(kThreads, 3) dequantize_heads_kernel(PoolArgs a) {
     extern __shared__ __align__(128) uint8_t smem[];

@@ -47,7 +47,7 @@
 // 5,500 waiting on P0 and P1 (96 MMAs then, 48 now), 2,200 a triangular solve for W, 1,500
 // the outputs. It takes 7,700 now, of which 2,200 are T and 1,250 A and Bm (both wait on
 // P0, 900, which follows P2, 1,100) and 900 R, PW and W.
-// 128 slots x 32 heads x 512 tokens: 4.05 ms then, 1.74 ms now.
+// 128 slots x 32 heads x 512 tokens: 4.05 ms then, 1.75 ms now.
 //
 // Hand-over, all by mbarriers, one phase a chunk, every wait bounded: `full1` (warps
 // 8-15: Q~, K~, K^, V, beta, g_C) starts P0, which completes `p0`; `ready` (warps 0-7: S,

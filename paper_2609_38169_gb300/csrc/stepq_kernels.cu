@@ -473,7 +473,7 @@ __global__ void __launch_bounds__(kThreads, 2) quantize_kernel(PoolArgs a) {
 // warp, its codes are read straight from the page and its 512 bytes leave as one
 // store instruction. (Staging the page in shared memory with 16 columns of a row per
 // thread wrote in 16-byte pieces 64 bytes apart and waited for the staging: 88 us for
-// 4096 heads at 6 bits, 54 us now; 47 us at the copy rate of HBM.)
+// 4096 heads at 6 bits, 51 us now; 47 us at the copy rate of HBM.)
 __global__ void __launch_bounds__(kThreads, 4) dequantize_kernel(PoolArgs a) {
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     const int b = blockIdx.x / a.heads, h = blockIdx.x - b * a.heads;
