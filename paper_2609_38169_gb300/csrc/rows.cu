@@ -195,7 +195,7 @@ __device__ __forceinline__ void issue(const DecodeArgs &a, const Smem &S, int h,
 // Slots are read and written in quads of four. Rows are stored by decreasing width, so all
 // but a few quads of a head hold integer rows of one width, each where the one before ends
 // (kQuad): addresses, shifts and masks are formed once for 16 codes. The width stays a
-// run-time value: with a body per width (a fifth fewer instructions again) the warps no
+// run-time value: with a body per width (a tenth fewer instructions still) the warps no
 // longer ran the same code, and waiting for it (no instruction: 0.5 -> 1.6 to 2.0 cycles
 // an issue) cost more than it gave. 256 sequences of 32 heads at 4 bits: 199 us so, 195 us
 // with every shift formed per row pair, 179 us here; four layers of 128 sequences at 6 bits:

@@ -677,7 +677,7 @@ __global__ void __launch_bounds__(kThreads, 2) distortion_kernel(DistArgs a) {
 // the fit's tile mapping (the replay's registers are reloaded from there).
 // Bound by the fits (three candidate widths plus FP16: about nine tenths of the
 // instructions at one sample in 8 tokens). 4 layers x 8 sequences x 32 heads, 256
-// tokens, 32 samples: 4.7 ms a pass, against about 28 ms of per-token launches.
+// tokens, 32 samples: 4.2 ms a pass, against about 28 ms of per-token launches.
 struct ReplayArgs {
     const float *k, *v, *beta, *gate;   // trace [L][T][n][..]
     const float *w;                     // [L][Hv][128]
