@@ -142,7 +142,8 @@ stepq_status launch_calib_observe(const stepq_config *cfg, int layers, const flo
 // stepq_kernels.cu: the FP32 replay of a trace with its candidate distortions, all layers
 stepq_status launch_calib_replay(const stepq_config *cfg, int n, int T, int every, const float *k,
                                  const float *v, const float *beta, const float *gate, const float *w,
-                                 const uint8_t *pivot_rows, double *acc, cudaStream_t s);
+                                 const uint8_t *pivot_rows, double *acc, const int32_t *heads, int n_heads,
+                                 cudaStream_t s);
 stepq_status launch_calib_distortion(const stepq_config *cfg, int layer, const float *w,
                                      const uint8_t *pivot_rows, const float *states, int n,
                                      double *acc, cudaStream_t s);

@@ -677,13 +677,14 @@ __global__ void __launch_bounds__(kThreads, 2) distortion_kernel(DistArgs a) {
 // the fit's tile mapping (the replay's registers are reloaded from there).
 // Bound by the fits (three candidate widths plus FP16: about nine tenths of the
 // instructions at one sample in 8 tokens). 4 layers x 8 sequences x 32 heads, 256
-// tokens, 32 samples: 4.2 ms a pass, against about 28 ms of per-token launches.
+// tokens, 32 samples: 4.2 ms a pass over all heads, against about 28 ms of per-token launches.
 struct ReplayArgs {
     const float *k, *v, *beta, *gate;   // trace [L][T][n][..]
     const float *w;                     // [L][Hv][128]
     const uint8_t *pivot_rows;          // [L][Hv][128] or null
     double *acc;                        // [L][Hv or Hv*128][K+1]
-    int n, T, Hk, Hv, every, gate_per_row;
+    const int32_t *heads;               // the heads to replay, layer * Hv + head, or null: all
+    int n_heads, n, T, Hk, Hv, every, gate_per_row;
     FitCands fit;
 };
 
@@ -705,9 +706,10 @@ __global__ void __launch_bounds__(kThreads, 2) replay_kernel(ReplayArgs a) {
     float2 *rowB = (float2 *)(smem + kRpRowB);
     double *acc = (double *)(smem + kRpAcc);
     const int tid = L.tid, w = L.warp, l = L.lane;
-    const int h = blockIdx.x % a.Hv, sb = blockIdx.x / a.Hv, b = sb % a.n, layer = sb / a.n;
+    const int at = blockIdx.x % a.n_heads, b = blockIdx.x / a.n_heads;
+    const size_t lh = a.heads ? a.heads[at] : at;
+    const int layer = (int)(lh / a.Hv), h = (int)(lh % a.Hv);
     const int hk = h / (a.Hv / a.Hk), K1 = a.fit.n_cand + 1;
-    const size_t lh = (size_t)layer * a.Hv + h;
     load_weights(L, S, a.w + lh * 128);
     for (int e = tid; e < 128 * K1; e += kThreads) acc[e] = 0.0;
     // A token's vectors: loaded two tokens ahead by threads 0..127 (one channel
@@ -890,14 +892,15 @@ stepq_status launch_calib_distortion(const stepq_config *cfg, int layer, const f
 
 stepq_status launch_calib_replay(const stepq_config *cfg, int n, int T, int every, const float *k,
                                  const float *v, const float *beta, const float *gate, const float *w,
-                                 const uint8_t *pivot_rows, double *acc, cudaStream_t s) {
+                                 const uint8_t *pivot_rows, double *acc, const int32_t *heads, int n_heads,
+                                 cudaStream_t s) {
     static SmemOptIn opt;
     const stepq_status st = opt((const void *)replay_kernel, kRpSmem);
     if (st != STEPQ_OK) return st;
     const bool rows = cfg->gate_kind == STEPQ_GATE_CHANNEL;
-    ReplayArgs a{k, v, beta, gate, w, rows ? pivot_rows : nullptr, acc, n, T, cfg->n_key_heads,
-                 cfg->n_value_heads, every, rows, fit_cands(cfg)};
-    const size_t ctas = (size_t)cfg->n_layers * n * cfg->n_value_heads;
+    ReplayArgs a{k, v, beta, gate, w, rows ? pivot_rows : nullptr, acc, heads, n_heads, n, T,
+                 cfg->n_key_heads, cfg->n_value_heads, every, rows, fit_cands(cfg)};
+    const size_t ctas = (size_t)n * n_heads;
     if (ctas > 0x7fffffffu) return STEPQ_ERR_UNSUPPORTED;
     replay_kernel<<<(unsigned)ctas, kThreads, kRpSmem, s>>>(a);
     return launched();

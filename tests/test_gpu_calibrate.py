@@ -21,6 +21,7 @@ def torch():
     ("tiny", 1, 4, 4, 1, 1, 1, 1, 0),          # one token, one sample
     ("gqa", 2, 2, 6, 3, 37, 5, 2, 1),          # ragged tail, three value heads a key head
     ("channel", 2, 3, 3, 2, 21, 4, 1, 9),      # pivot rows: the second pass
+    ("channel", 2, 3, 3, 2, 21, 4, 1, 2),      # pivot rows in some heads only
     ("channel", 1, 1, 2, 5, 64, 64, 2, 0),     # a single sample at the end
 ])
 def test_calibration_equals_token_steps(torch, name, layers, hk, hv, n, T, every, iters, pivots):
