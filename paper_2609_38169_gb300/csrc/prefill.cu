@@ -15,12 +15,12 @@
 //
 // Every product runs on the tensor cores (tcgen05, kind::tf32) in split
 // precision: an fp32 operand is its TF32 head, which is all the tensor core reads of
-// it, plus a remainder, and a product is head*head + head*rest + rest*head (P0 and P1
+// it, plus a remainder, and a product is head*head + head*rest + rest*head (P0 and PW
 // also take rest*rest), which keeps fp32 accuracy. The state stays in tensor memory as
 // S^T (lane j = value column, column i = key row):
 //   P0  [Q~ ; K~] K^T        -> Bm, A      M = 128, N = 64, K = 128, A, B in smem
 //   P1  S_0^T [Q~ ; K~]^T    -> [Q~ S_0 ; K~ S_0]^T    M = 128, N = 128 / 64, K = 128, A in tmem
-//   PW  W^T = R^T T^T, T = (I + A)^-1, R = diag(beta) (V - K~ S_0)   M = 128, N = 64 / 32, K = 32
+//   PW  W^T - R^T = R^T (T - I)^T, T = (I + A)^-1, R = diag(beta) (V - K~ S_0)   M = 128, N = 64, K = 32
 //   P2  S^T += W^T K_bar and Y^T = (Q~ S_0)^T + W^T Bm^T   M = 128, N = 160, K = 32, A in tmem
 // An MMA with M = 128 takes N / 2 cycles, but not less than the 35 to 45 that its issue
 // takes, so operands are stacked until N is 128 where they can be: P0's A rows and P1's B
@@ -29,6 +29,17 @@
 // of stacked rests land in columns (or, P0, lanes) of their own and are added when they
 // are read. Shared-memory operands are K-major core matrices (8 rows x 16 bytes). The
 // FMA pipe keeps the element-wise work, the inverse T and the scaling of S by g_C.
+//
+// Precision of W: the identity's part of T R is R itself, added in fp32, so that only
+// (T - I) R goes through split operands; the rests of R and W are rounded, not truncated,
+// to what the tensor core keeps of them; and the lower blocks of T are formed as
+// T22 (N21 T11), the order whose rounding T11 does not amplify. W then is as near to fp64 as
+// by a forward substitution in fp32 or nearer (0.7 to 0.96 of its error with keys from
+// random to equal and beta up to 1; W = T R from truncated rests: 1.2 to 1.5). Whole outputs,
+// 512 tokens, random keys, scalar gates 0.85 to 0.999: y 1.08e-6 and the final state 4.4e-7
+// off, at 1.76 ms as below; with W = T R 1.30e-6 and 6.7e-7 at 1.75 ms; with the substitution,
+// P0 without rest*rest, 1.88e-6 and 5.8e-7. (The state's rest rounded too gives 1.05e-6 and
+// 4.4e-7, but lies on the chain: 1.82 ms.)
 //
 // One persistent CTA of 20 warps per SM; it owns all 512 tensor-memory columns:
 //   [0, 128) S^T | [128, 160) Y^T | [160, 192) (K~ S_0)^T, then R^T | [192, 256) the rests'
@@ -47,7 +58,7 @@
 // 5,500 waiting on P0 and P1 (96 MMAs then, 48 now), 2,200 a triangular solve for W, 1,500
 // the outputs. It takes 7,700 now, of which 2,200 are T and 1,250 A and Bm (both wait on
 // P0, 900, which follows P2, 1,100) and 900 R, PW and W.
-// 128 slots x 32 heads x 512 tokens: 4.05 ms then, 1.75 ms now.
+// 128 slots x 32 heads x 512 tokens: 4.05 ms then, 1.76 ms now.
 //
 // Hand-over, all by mbarriers, one phase a chunk, every wait bounded: `full1` (warps
 // 8-15: Q~, K~, K^, V, beta, g_C) starts P0, which completes `p0`; `ready` (warps 0-7: S,
@@ -76,7 +87,7 @@ constexpr uint32_t kColS = 0, kColY = 128, kColX = 160, kColYl = 192, kColXl = 2
 constexpr uint32_t kCols = 512;
 constexpr uint32_t kIdescP0 = tc::idesc_tf32(128, 64);
 constexpr uint32_t kIdescP1 = tc::idesc_tf32(128, 128), kIdescP1l = tc::idesc_tf32(128, 64);
-constexpr uint32_t kIdescPw = tc::idesc_tf32(128, 64), kIdescPwl = tc::idesc_tf32(128, 32);
+constexpr uint32_t kIdescPw = tc::idesc_tf32(128, 64);
 constexpr uint32_t kIdescP2 = tc::idesc_tf32(128, 160);
 
 // Shared-memory operands: K-major core matrices of 8 rows x 4 fp32 (128 B). Strides are
@@ -369,7 +380,7 @@ __device__ __forceinline__ bool issue_mma(const Args &a, uint8_t *smem, uint64_t
 #pragma unroll
         for (int s = 0; s < 4; s++) {
             tc::mma_tf32_ts(lead, tm + kColW, tm + kColX + 8 * s, dT + s * k32, kIdescPw, s > 0 ? 1u : 0u);
-            tc::mma_tf32_ts(lead, tm + kColW, tm + kColXl + 8 * s, dT + s * k32, kIdescPwl, 1u);
+            tc::mma_tf32_ts(lead, tm + kColW, tm + kColXl + 8 * s, dT + s * k32, kIdescPw, 1u);
         }
         tc::commit(lead, &bars[kPw]);
         if (!(ok = wait(kFull2, ph) && wait(kWready, ph))) break;
@@ -389,7 +400,7 @@ __device__ __forceinline__ bool issue_mma(const Args &a, uint8_t *smem, uint64_t
 
 // Warp 17: T = (I + A)^-1 of every chunk from N = -A, by blocks: the 8 x 8 diagonal
 // blocks by substitution (a row per lane), then the lower parts of the 16 x 16 and the
-// 32 x 32 blocks as (T22 N21) T11, two dense products each. One substitution over 32 rows
+// 32 x 32 blocks as T22 (N21 T11), two dense products each. One substitution over 32 rows
 // is a chain of 31 dependent steps (2,400 cycles or more; this takes 2,200 beside the
 // other warps' shared-memory traffic). A lane holds a row of the
 // left factor and reads the right one's rows, 16 bytes at a time, eight loads in flight.
@@ -452,11 +463,11 @@ __device__ __forceinline__ bool invert(const Args &a, uint8_t *smem, uint64_t *b
             const int o = l & 16, r = l & 7, c = 4 * ((l >> 3) & 1);
             float *v = T + ((o >> 1) + r) * kMRow + 16;               // in T's zero part
             uint64_t lo = 0, hi = 0;
-            row8(T + (o + 8 + r) * kMRow + o + 8, N + (o + 8) * kMRow + o + c, lo, hi);
+            row8(N + (o + 8 + r) * kMRow + o, T + o * kMRow + o + c, lo, hi);
             put(v + c, lo, hi);
             __syncwarp();
             lo = hi = 0;
-            row8(v, T + o * kMRow + o + c, lo, hi);
+            row8(T + (o + 8 + r) * kMRow + o + 8, v - r * kMRow + c, lo, hi);
             put(T + (o + 8 + r) * kMRow + o + c, lo, hi);
         }
         __syncwarp();
@@ -466,8 +477,8 @@ __device__ __forceinline__ bool invert(const Args &a, uint8_t *smem, uint64_t *b
             uint64_t y[4] = {0, 0, 0, 0};
 #pragma unroll
             for (int s = 0; s < 16; s += 8) {
-                row8(T + (16 + r) * kMRow + 16 + s, N + (16 + s) * kMRow + c, y[0], y[1]);
-                row8(T + (16 + r) * kMRow + 16 + s, N + (16 + s) * kMRow + c + 4, y[2], y[3]);
+                row8(N + (16 + r) * kMRow + s, T + s * kMRow + c, y[0], y[1]);
+                row8(N + (16 + r) * kMRow + s, T + s * kMRow + c + 4, y[2], y[3]);
             }
             put(v + c, y[0], y[1]);
             put(v + c + 4, y[2], y[3]);
@@ -475,19 +486,19 @@ __device__ __forceinline__ bool invert(const Args &a, uint8_t *smem, uint64_t *b
             y[0] = y[1] = y[2] = y[3] = 0;
 #pragma unroll
             for (int s = 0; s < 16; s += 8) {
-                row8(v + s, T + s * kMRow + c, y[0], y[1]);
-                row8(v + s, T + s * kMRow + c + 4, y[2], y[3]);
+                row8(T + (16 + r) * kMRow + 16 + s, T + s * kMRow + 16 + c, y[0], y[1]);
+                row8(T + (16 + r) * kMRow + 16 + s, T + s * kMRow + 16 + c + 4, y[2], y[3]);
             }
             put(T + (16 + r) * kMRow + c, y[0], y[1]);
             put(T + (16 + r) * kMRow + c + 4, y[2], y[3]);
         }
         __syncwarp();
-        // The operand: row t = lane, zero above the diagonal.
+        // The operand T - I: row t = lane, zero from the diagonal on.
 #pragma unroll
         for (int s = 0; s < C; s += 4) {
             const float4 x = *(const float4 *)(T + l * kMRow + s);
             put4(smem + kOffT, smem + kOffTl, off32(l, s),
-                 make_float4(s <= l ? x.x : 0.f, s + 1 <= l ? x.y : 0.f, s + 2 <= l ? x.z : 0.f, s + 3 <= l ? x.w : 0.f));
+                 make_float4(s < l ? x.x : 0.f, s + 1 < l ? x.y : 0.f, s + 2 < l ? x.z : 0.f, s + 3 < l ? x.w : 0.f));
         }
         fence_async_smem();
         mbar_arrive(&bars[kT]);
@@ -603,17 +614,18 @@ __device__ __forceinline__ bool chain(const Args &a, uint8_t *smem, uint64_t *ba
             // in the place of K~ S_0 and its rest.
             ok = mbar_wait(&bars[kP1], ph, pipe::kWaitCycles);
             tc::fence_after();
+            float r[16];                                  // W = R + (T - I) R takes R again
             {
-                float x[16], xl[16];
-                tc::ld16(tl + kColX + 16 * half, x);
+                float xl[16];
+                tc::ld16(tl + kColX + 16 * half, r);
                 tc::ld16(tl + kColXl + 16 * half, xl);
 #pragma unroll
                 for (int e = 0; e < 16; e++) {
                     const int t = 16 * half + e;
-                    x[e] = bet[t] * (V[t * 128 + (j ^ 4 * (t & 7))] - (x[e] + xl[e]));
-                    xl[e] = tc::tf32_rest(x[e]);
+                    r[e] = bet[t] * (V[t * 128 + (j ^ 4 * (t & 7))] - (r[e] + xl[e]));
+                    xl[e] = tc::tf32_rest_rn(r[e]);
                 }
-                tc::st16(tl + kColX + 16 * half, x);
+                tc::st16(tl + kColX + 16 * half, r);
                 tc::st16(tl + kColXl + 16 * half, xl);
             }
             tc::wait_st();
@@ -641,8 +653,8 @@ __device__ __forceinline__ bool chain(const Args &a, uint8_t *smem, uint64_t *ba
                 tc::ld16(tl + kColWl + 16 * half, xl);
 #pragma unroll
                 for (int e = 0; e < 16; e++) {
-                    x[e] += xl[e];
-                    xl[e] = tc::tf32_rest(x[e]);
+                    x[e] = r[e] + (x[e] + xl[e]);
+                    xl[e] = tc::tf32_rest_rn(x[e]);
                 }
                 tc::st16(tl + kColW + 16 * half, x);
                 tc::st16(tl + kColWl + 16 * half, xl);

@@ -207,6 +207,11 @@ __device__ __forceinline__ void wait_st() { asm volatile("tcgen05.wait::st.sync.
 // tensor or shared memory, with its low 13 mantissa bits cleared (checked on GB300:
 // 1024 of 1024 values of each kind truncated), so x itself serves as the head.
 __device__ __forceinline__ float tf32_rest(float x) { return x - __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
+// The same, rounded to nearest in what the tensor core will keep of it: its 13 bits are
+// cut to 11, by truncation an error of up to 2^-21 of x and always towards zero.
+__device__ __forceinline__ float tf32_rest_rn(float x) {
+    return __uint_as_float(__float_as_uint(tf32_rest(x)) + 0x1000u);
+}
 
 // ---- registers: a warpgroup's share of the CTA's registers (executed by all its warps;
 // the shares may not add up to more than the launch's total) ----
