@@ -49,13 +49,13 @@ int sm_count() {
 
 stepq_status SmemOptIn::operator()(const void *kernel, int bytes) {
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return STEPQ_ERR_CUDA;
+    stepq_status st = cuda_status(cudaGetDevice(&dev));
+    if (st != STEPQ_OK || dev < 0 || dev >= kMaxDevices) return STEPQ_ERR_CUDA;
     const uint64_t bit = 1ull << dev;
     if (done.load(std::memory_order_acquire) & bit) return STEPQ_OK;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess)
-        return STEPQ_ERR_CUDA;
-    done.fetch_or(bit, std::memory_order_release);
-    return STEPQ_OK;
+    st = cuda_status(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    if (st == STEPQ_OK) done.fetch_or(bit, std::memory_order_release);
+    return st;
 }
 
 // The pipelined kernels' wait bound and withheld item (test support). Plain

@@ -154,6 +154,15 @@ stepq_status launch_validate_slots_static(const int32_t *slots, int B, int pool_
 stepq_status read_device_error(cudaStream_t s);
 int sm_count();                      // multiprocessors of the current device
 
+// Status of a runtime call that returns its error. The error is taken from the runtime
+// too: left there, it would fail the next launch that is checked by cudaGetLastError(),
+// this library's or the caller's.
+inline stepq_status cuda_status(cudaError_t e) {
+    if (e == cudaSuccess) return STEPQ_OK;
+    cudaGetLastError();
+    return STEPQ_ERR_CUDA;
+}
+
 // Launch of a kernel that may overlap the end of the stream's previous kernel: its
 // CTAs take their places, and run up to griddep_wait(), as that kernel's CTAs leave.
 // A decode launch spends about 3 us before its first page arrives (placing the
@@ -172,7 +181,7 @@ inline stepq_status launch_overlapped(void (*kernel)(Args, Rest...), int grid, i
     at[0].val.programmaticStreamSerializationAllowed = 1;
     c.attrs = at;
     c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, kernel, a, rest...) == cudaSuccess ? STEPQ_OK : STEPQ_ERR_CUDA;
+    return cuda_status(cudaLaunchKernelEx(&c, kernel, a, rest...));
 }
 
 constexpr int kSmemMax = 227 * 1024;   // dynamic shared memory one CTA can have
