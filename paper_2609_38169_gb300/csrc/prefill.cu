@@ -760,11 +760,14 @@ stepq_status launch_prefill(const stepq_config *cfg, const float *q, const float
     const stepq_status st = opt((const void *)pf::prefill_kernel, pf::kSmem);
     if (st != STEPQ_OK) return st;
     // the register shares are taken from what the kernel is launched with
-    static const int regs = [] {
+    static std::atomic<int> regs{0};                       // kept once known
+    if (regs.load(std::memory_order_relaxed) == 0) {
         cudaFuncAttributes f{};
-        return cudaFuncGetAttributes(&f, (const void *)pf::prefill_kernel) == cudaSuccess ? f.numRegs : 0;
-    }();
-    if (regs < pf::kRegs) return STEPQ_ERR_CUDA;
+        const stepq_status e = cuda_status(cudaFuncGetAttributes(&f, (const void *)pf::prefill_kernel));
+        if (e != STEPQ_OK) return e;
+        regs.store(f.numRegs, std::memory_order_relaxed);
+    }
+    if (regs.load(std::memory_order_relaxed) < pf::kRegs) return STEPQ_ERR_CUDA;
     int grid = sm_count();
     if (grid > a.items) grid = a.items;
     return launch_overlapped(pf::prefill_kernel, grid, pf::kBlock, pf::kSmem, s, a);

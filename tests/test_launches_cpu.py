@@ -77,3 +77,13 @@ for name, call in calls.items():
     assert calls["observe"]() == 0, name           # a plain launch, checked by the last error
     assert call() == 0, name
 """)
+
+
+def test_prefill_after_a_failed_attribute_query(run):
+    """A failed query of prefill's register count fails that call alone."""
+    run(f"""
+fake.fake_refuse({GET_ATTRIBUTES}, 1)
+assert calls["prefill"]() == {STEPQ_ERR_CUDA}
+assert fake.fake_pending_error() == 0 and fake.fake_launches() == 0
+assert calls["observe"]() == 0 and calls["prefill"]() == 0
+""")
