@@ -630,7 +630,7 @@ __global__ void __launch_bounds__(kThreads, 2) decode_heads_kernel(DecodeArgs a)
     }
     __syncthreads();
     griddep_wait();
-    griddep_launch();
+    if (MODE != kReadout) griddep_launch();                // a readout: as its CTAs end (launch_overlapped)
     const pipe::Shape p{a.items, a.nb, a.n_stages, a.slots, a.pool_slots, a.err, a.stall.wait_cycles,
                         a.stall.withhold_item};
     pipe::run(
