@@ -360,12 +360,12 @@ stepq_status stepq_device_error(stepq_stream_t stream);
 stepq_status stepq_stream_status(stepq_stream_t stream);
 
 /* Test support for the bounded waits (not for production use). Every wait of
- * the pipelined decode kernels (stepq_decode_step, the split halves, the FP32
- * and INT-b decode steps) gives up after `wait_cycles` SM clock cycles
+ * the pipelined kernels (stepq_decode_step, the split halves, the FP32 and INT-b
+ * decode steps, stepq_prefill_fp32) gives up after `wait_cycles` SM clock cycles
  * (default 2e9, about one second; at least 1000), raises STEPQ_ERR_TIMEOUT and
  * lets its CTA return. withhold_item >= 0 makes every later launch skip the
- * copies of that item (head * B + batch entry), so that its wait runs out and
- * the launch reports STEPQ_ERR_TIMEOUT with its results undefined; -1 restores
+ * copies of that item (head * B + batch entry; prefill: the first copies of batch
+ * entry * Hv + head), so that its wait runs out and the launch reports STEPQ_ERR_TIMEOUT with its results undefined; -1 restores
  * normal operation. The values are process-wide, read at each launch, and not
  * safe to change while another thread launches. STEPQ_ERR_ARG for values out of
  * range. The paper has no counterpart; this exists to test failure detection. */

@@ -70,7 +70,6 @@
 #include "async.cuh"
 #include "device.cuh"
 #include "internal.h"
-#include "pipeline.cuh"
 #include "tcgen05.cuh"
 
 namespace stepq {
@@ -157,8 +156,9 @@ __device__ __forceinline__ bool group_any(bool p) {
 struct Args {
     const float *q, *k, *v, *beta, *gate;
     float *states, *y;
-    int B, T, Hk, Hv, gate_per_row, items;
+    int B, T, Hk, Hv, gate_per_row, items;   // item = batch entry * Hv + head
     unsigned int *err;
+    StallKnob stall;
 };
 
 // Cumulative gates of a chunk: this thread's float4 of four channels at tokens 8 m + tl
@@ -230,7 +230,7 @@ __device__ __forceinline__ bool produce(const Args &a, uint8_t *smem, uint64_t *
         return t < fn ? *(const float4 *)(p + t * kQRow) : make_float4(0.f, 0.f, 0.f, 0.f);
     };
     const auto wait = [&](int bar, uint32_t ph) {
-        return (bool)__all_sync(0xffffffffu, mbar_wait(&bars[bar], ph, pipe::kWaitCycles));
+        return (bool)__all_sync(0xffffffffu, mbar_wait(&bars[bar], ph, a.stall.wait_cycles));
     };
     int item = blockIdx.x, c0 = 0;
     if (item < a.items) {
@@ -324,8 +324,9 @@ __device__ __forceinline__ bool load_qk(const Args &a, uint8_t *smem, uint64_t *
     for (int item = blockIdx.x; ok && item < a.items; item += gridDim.x) {
         const int b = item / a.Hv, hk = (item - b * a.Hv) / grp;
         for (int c0 = 0; c0 < a.T; c0 += C, n++) {
-            ok = n == 0 || __all_sync(0xffffffffu, mbar_wait(&bars[kFull1], (n - 1) & 1u, pipe::kWaitCycles));
+            ok = n == 0 || __all_sync(0xffffffffu, mbar_wait(&bars[kFull1], (n - 1) & 1u, a.stall.wait_cycles));
             if (!ok) break;
+            if (item == a.stall.withhold_item && c0 == 0) continue;   // test switch: these copies never start
             const int tokens = min(C, a.T - c0);
             if (l == 0) mbar_arrive_tx(&bars[kIn], (uint32_t)tokens * 1024u);
             __syncwarp();
@@ -337,7 +338,7 @@ __device__ __forceinline__ bool load_qk(const Args &a, uint8_t *smem, uint64_t *
         }
     }
     // no copy is in flight when the CTA ends, whatever stalled
-    return (n == 0 || mbar_wait(&bars[kIn], (n - 1) & 1u, pipe::kWaitCycles)) && ok;
+    return (n == 0 || mbar_wait(&bars[kIn], (n - 1) & 1u, a.stall.wait_cycles)) && ok;
 }
 
 // Warp 16: the MMAs of this CTA's chunks, issued by one elected lane; the whole warp runs
@@ -352,7 +353,7 @@ __device__ __forceinline__ bool issue_mma(const Args &a, uint8_t *smem, uint64_t
     const long long chunks = (long long)per * mine;
     const uint32_t lead = tc::elect();
     const auto wait = [&](int bar, uint32_t ph) {
-        const bool ok = __all_sync(0xffffffffu, mbar_wait(&bars[bar], ph, pipe::kWaitCycles));
+        const bool ok = __all_sync(0xffffffffu, mbar_wait(&bars[bar], ph, a.stall.wait_cycles));
         tc::fence_after();
         return ok;
     };
@@ -431,7 +432,7 @@ __device__ __forceinline__ bool invert(const Args &a, uint8_t *smem, uint64_t *b
     };
     for (long long n = 0; n < chunks; n++) {
         const uint32_t ph = (uint32_t)n & 1u;
-        if (!__all_sync(0xffffffffu, mbar_wait(&bars[kA], ph, pipe::kWaitCycles))) return false;
+        if (!__all_sync(0xffffffffu, mbar_wait(&bars[kA], ph, a.stall.wait_cycles))) return false;
         {   // 8 x 8 blocks: lane 8 b + r holds row r of block b
             const int o = l & 24, r = l & 7;
             const float *m = N + o * kMRow + o;
@@ -543,7 +544,7 @@ __device__ __forceinline__ bool chain(const Args &a, uint8_t *smem, uint64_t *ba
             const float *gC = (const float *)(smem + kOffGc) + ph * 128;
             const float *bet = (const float *)(smem + kOffBeta) + ph * C;
             // full1 first: its next phase then cannot end before this thread has seen this one
-            ok = mbar_wait(&bars[kFull1], ph, pipe::kWaitCycles) && ok;
+            ok = mbar_wait(&bars[kFull1], ph, a.stall.wait_cycles) && ok;
             if (t0 == 0) tc::wait_st();
             tc::fence_before();
             mbar_arrive(&bars[kReady]);
@@ -560,7 +561,7 @@ __device__ __forceinline__ bool chain(const Args &a, uint8_t *smem, uint64_t *ba
             // P0's result, row r = lane: [Q~ ; K~] in lanes 0-63, its rests in 64-127;
             // columns s over K^, 32 + s over its rests. This half takes columns
             // 16 half .. +15.
-            ok = mbar_wait(&bars[kP0], ph, pipe::kWaitCycles) && ok;
+            ok = mbar_wait(&bars[kP0], ph, a.stall.wait_cycles) && ok;
             tc::fence_after();
             float d[16];
             {
@@ -612,7 +613,7 @@ __device__ __forceinline__ bool chain(const Args &a, uint8_t *smem, uint64_t *ba
             store_y();
             // R = diag(beta) (V - K~ S_0), tokens 16 half .. +15 of column j, and its rest,
             // in the place of K~ S_0 and its rest.
-            ok = mbar_wait(&bars[kP1], ph, pipe::kWaitCycles);
+            ok = mbar_wait(&bars[kP1], ph, a.stall.wait_cycles);
             tc::fence_after();
             float r[16];                                  // W = R + (T - I) R takes R again
             {
@@ -645,7 +646,7 @@ __device__ __forceinline__ bool chain(const Args &a, uint8_t *smem, uint64_t *ba
                 }
                 tc::st64(tl + kColS + 64 * half, sv);
             }
-            ok = mbar_wait(&bars[kPw], ph, pipe::kWaitCycles) && ok;
+            ok = mbar_wait(&bars[kPw], ph, a.stall.wait_cycles) && ok;
             tc::fence_after();
             {
                 float x[16], xl[16];
@@ -662,7 +663,7 @@ __device__ __forceinline__ bool chain(const Args &a, uint8_t *smem, uint64_t *ba
             tc::wait_st();
             tc::fence_before();
             mbar_arrive(&bars[kWready]);
-            ok = mbar_wait(&bars[kP2], ph, pipe::kWaitCycles) && ok;
+            ok = mbar_wait(&bars[kP2], ph, a.stall.wait_cycles) && ok;
             tc::fence_after();
             // Outputs: tokens 16 half .. 16 half + 15 of column j, stored once the next
             // chunk can start.
@@ -756,6 +757,7 @@ stepq_status launch_prefill(const stepq_config *cfg, const float *q, const float
     a.gate_per_row = cfg->gate_kind == STEPQ_GATE_CHANNEL;
     a.items = B * a.Hv;
     a.err = device_error_word();
+    a.stall = stall_knob();
     static SmemOptIn opt;
     const stepq_status st = opt((const void *)pf::prefill_kernel, pf::kSmem);
     if (st != STEPQ_OK) return st;
