@@ -13,7 +13,7 @@ namespace stepq {
 
 struct ObsArgs {
     const float *q, *k, *beta, *gate;      // [layers][n][..]
-    int n, layers, Hk, Hv, gate_per_row, chunk;
+    int n, Hk, Hv, gate_per_row, chunk;
     double *omega, *logret;                // sums: [layers][Hv][128], [layers][Hv] or [layers][Hv][128]
     double *part;                          // chunk partials [chunks][layers][Hv][256], or null
 };
@@ -112,7 +112,6 @@ stepq_status launch_calib_observe(const stepq_config *cfg, int layers, const flo
     ObsArgs a{};
     a.q = q; a.k = k; a.beta = beta; a.gate = gate;
     a.n = n;
-    a.layers = layers;
     a.Hk = cfg->n_key_heads;
     a.Hv = cfg->n_value_heads;
     a.gate_per_row = cfg->gate_kind == STEPQ_GATE_CHANNEL;

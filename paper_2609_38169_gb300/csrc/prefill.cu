@@ -156,7 +156,7 @@ __device__ __forceinline__ bool group_any(bool p) {
 struct Args {
     const float *q, *k, *v, *beta, *gate;
     float *states, *y;
-    int B, T, Hk, Hv, gate_per_row, items;   // item = batch entry * Hv + head
+    int T, Hk, Hv, gate_per_row, items;      // item = batch entry * Hv + head
     unsigned int *err;
     StallKnob stall;
 };
@@ -751,7 +751,7 @@ stepq_status launch_prefill(const stepq_config *cfg, const float *q, const float
     pf::Args a{};
     a.q = q; a.k = k; a.v = v; a.beta = beta; a.gate = gate;
     a.states = states; a.y = y;
-    a.B = B; a.T = T;
+    a.T = T;
     a.Hk = cfg->n_key_heads;
     a.Hv = cfg->n_value_heads;
     a.gate_per_row = cfg->gate_kind == STEPQ_GATE_CHANNEL;

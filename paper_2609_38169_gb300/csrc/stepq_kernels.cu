@@ -344,10 +344,6 @@ __device__ __forceinline__ void load_dense(const Lane &L, const float *X, uint64
     }
 }
 
-__device__ __forceinline__ void copy16(uint4 *dst, const uint4 *src, int n16, int tid) {
-    for (int e = tid; e < n16; e += kThreads) dst[e] = src[e];
-}
-
 // ---------------------------------------------------------- quantize / dequantize
 struct PoolArgs {
     uint8_t *pool;
