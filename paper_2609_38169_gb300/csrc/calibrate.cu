@@ -43,9 +43,10 @@ struct Workspace {
         w = (float *)take(heads * kD * sizeof(float));
         pivot = take(U);
         // About 16 observe CTAs per SM, within the size of n dense states of a layer.
+        // (The bytes asked for do not depend on the device.)
         const size_t most = std::max<size_t>(1, 32 * (size_t)n / cfg->n_layers);
-        chunks = (int)std::min(most, (16 * 152 + heads - 1) / heads);
-        scratch = base && chunks > 1 ? (double *)(base + o) : nullptr;
+        chunks = base ? (int)std::min(most, (16 * (size_t)sm_count() + heads - 1) / heads) : 1;
+        scratch = chunks > 1 ? (double *)(base + o) : nullptr;
         // The size is part of the interface, in what is asked for and in what is refused:
         // n slot ids, n dense states and n readouts of a layer, as when the replay went
         // through memory.
