@@ -56,7 +56,7 @@
 //   warp 18     q and k of the next chunk by bulk copies
 // With 8 warps doing all of it in turn a chunk took 17,700 cycles: 6,700 the operands,
 // 5,500 waiting on P0 and P1 (96 MMAs then, 48 now), 2,200 a triangular solve for W, 1,500
-// the outputs. It takes 7,700 now, of which 2,200 are T and 1,250 A and Bm (both wait on
+// the outputs. It takes 7,800 now, of which 2,200 are T and 1,250 A and Bm (both wait on
 // P0, 900, which follows P2, 1,100) and 900 R, PW and W.
 // 128 slots x 32 heads x 512 tokens: 4.05 ms then, 1.76 ms now.
 //

@@ -364,7 +364,7 @@ struct PoolArgs {
 // refilled with the next item's state (16-byte cp.async, swizzled as cgroup), and the
 // page leaves by a bulk store. One CTA per item with plain loads exposed their
 // latency (stalled on it 18% of the time at 24% occupancy): 4096 heads at 6 bits
-// took 143 us, 110 us now (47 us at the copy rate of HBM).
+// took 143 us, 109 us now (47 us at the copy rate of HBM).
 constexpr int kQTile = 0;                                    // float [128][128], 16-byte groups swizzled
 constexpr int kQPage = kN * 4;
 constexpr int kQFit = kQPage + (int)kMaxHeadBytes;

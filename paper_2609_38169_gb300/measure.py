@@ -97,8 +97,8 @@ def prefill(slots=128, tokens=512, name="gqa"):
     head_tokens = slots * tokens * wl.hv
     C = 32
     # tensor-core work issued per chunk of one head (TF32 heads and rests stacked along N):
-    # P0 128 x 64 x 128, P1 128 x (128 + 64) x 128, PW 128 x (64 + 32) x 32, P2 3 x 128 x 160 x 32
-    mma_flops = 2 * 128 * ((64 + 192) * 128 + (96 + 3 * 160) * 32) / C
+    # P0 128 x 64 x 128, P1 128 x (128 + 64) x 128, PW 2 x 128 x 64 x 32, P2 3 x 128 x 160 x 32
+    mma_flops = 2 * 128 * ((64 + 192) * 128 + (2 * 64 + 3 * 160) * 32) / C
     # the fp32 work of the chunkwise form per head-token: K~S, Q~S and the state
     # update (3 x 128 x 128 FMAs), A and Q~K^T (2 x C x 128), the solve and Bm W (1.5 x C x 128)
     fma = 3 * D * D + 2 * C * D + 1.5 * C * D
