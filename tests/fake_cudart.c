@@ -1,5 +1,5 @@
 // A CUDA runtime without a GPU, preloaded before libcudart: "device" memory is host
-// memory, launches are recorded instead of run, and calls can be made to fail. The
+// memory, launches are counted instead of run, and calls can be made to fail. The
 // last error is kept as the runtime keeps it: set by a failing call, returned and
 // cleared by cudaGetLastError().
 #include <stdlib.h>
@@ -7,11 +7,7 @@
 
 #include <cuda_runtime_api.h>
 
-#define MAX_KERNELS 128
-static const void *kernel_ptr[MAX_KERNELS];
-static const char *kernel_name[MAX_KERNELS];
-static int n_kernels, n_launches, last_overlapped;
-static const void *last_kernel;
+static int n_launches;
 static cudaError_t last_error;
 // calls of the kind still to be refused: 0 launches, 1 cudaFuncSetAttribute, 2 cudaFuncGetAttributes
 static int refuse[3];
@@ -25,13 +21,7 @@ static int refused(int kind) { return refuse[kind] > 0 && refuse[kind]-- > 0; }
 // ---- for the tests ----
 void fake_refuse(int kind, int times) { refuse[kind] = times; }
 int fake_launches(void) { return n_launches; }
-int fake_overlapped(void) { return last_overlapped; }
 int fake_pending_error(void) { return (int)last_error; }
-const char *fake_kernel(void) {
-    for (int i = 0; i < n_kernels; i++)
-        if (kernel_ptr[i] == last_kernel) return kernel_name[i];
-    return "";
-}
 
 // ---- the runtime's calls ----
 cudaError_t cudaGetLastError(void) {
@@ -83,27 +73,21 @@ cudaError_t cudaFuncGetAttributes(struct cudaFuncAttributes *a, const void *f) {
     a->numRegs = 96;
     return done(refused(2) ? cudaErrorInvalidValue : cudaSuccess);
 }
-static cudaError_t launch(const void *f, int overlapped) {
+static cudaError_t launch(void) {
     if (refused(0)) return done(cudaErrorInvalidConfiguration);
     n_launches++;
-    last_kernel = f;
-    last_overlapped = overlapped;
     return cudaSuccess;
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **args) {
-    int overlapped = 0;
-    (void)args;
-    for (unsigned i = 0; i < c->numAttrs; i++)
-        if (c->attrs[i].id == cudaLaunchAttributeProgrammaticStreamSerialization)
-            overlapped = c->attrs[i].val.programmaticStreamSerializationAllowed;
-    return launch(f, overlapped);
+    (void)c; (void)f; (void)args;
+    return launch();
 }
 
 // ---- what <<<>>> and the registration of a library's kernels turn into ----
 cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) { *k = (cudaKernel_t)f; return cudaSuccess; }
 cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3 block, void **args, size_t smem, cudaStream_t st) {
-    (void)grid; (void)block; (void)args; (void)smem; (void)st;
-    return launch((const void *)k, 0);
+    (void)k; (void)grid; (void)block; (void)args; (void)smem; (void)st;
+    return launch();
 }
 static dim3 pushed_grid, pushed_block;
 unsigned __cudaPushCallConfiguration(dim3 grid, dim3 block, size_t smem, void *st) {
@@ -124,11 +108,7 @@ void __cudaRegisterFatBinaryEnd(void **h) { (void)h; }
 void __cudaUnregisterFatBinary(void **h) { (void)h; }
 void __cudaRegisterFunction(void **h, const char *host, char *dev, const char *name, int limit, void *tid, void *bid,
                             void *bdim, void *gdim, int *wsize) {
-    (void)h; (void)dev; (void)limit; (void)tid; (void)bid; (void)bdim; (void)gdim; (void)wsize;
-    if (n_kernels < MAX_KERNELS) {
-        kernel_ptr[n_kernels] = host;
-        kernel_name[n_kernels++] = name;
-    }
+    (void)h; (void)host; (void)dev; (void)name; (void)limit; (void)tid; (void)bid; (void)bdim; (void)gdim; (void)wsize;
 }
 void __cudaRegisterVar(void **h, char *host, char *dev, const char *name, int ext, size_t size, int constant, int global) {
     (void)h; (void)host; (void)dev; (void)name; (void)ext; (void)size; (void)constant; (void)global;

@@ -16,7 +16,6 @@ import ctypes as C
 import numpy as np
 from paper_2609_38169_gb300 import api as A, _lib
 fake = C.CDLL(None)
-fake.fake_kernel.restype = C.c_char_p
 L, p, B = _lib.lib(), C.c_void_p(1 << 20), 4
 assert fake.fake_launches() == 0
 def plan_of(gate):
@@ -48,12 +47,11 @@ STEPQ_ERR_CUDA = 5
 
 @pytest.fixture(scope="module")
 def run(tmp_path_factory):
-    so = build_ext.build()
+    build_ext.build()
     cuda = os.path.dirname(os.path.dirname(os.path.realpath(build_ext.nvcc())))
     fake = str(tmp_path_factory.mktemp("fake") / "libfake.so")
     subprocess.run(["gcc", "-O1", "-shared", "-fPIC", "-Wall", "-I", os.path.join(cuda, "include"),
                     os.path.join(HERE, "fake_cudart.c"), "-o", fake], check=True)
-    assert os.path.exists(so)
 
     def child(code):
         r = subprocess.run([sys.executable, "-c", CALLS + code], cwd=os.path.dirname(HERE), capture_output=True,
